@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <numeric>
 #include <cmath>
 #include <cstdio>
@@ -23,6 +24,7 @@
 #include "dugks_adjoint_rows.cuh"
 #include "dugks_batch.cuh"
 #include "dugks_kernels.cuh"
+#include "dugks_resident.cuh"
 #include "dugks_step_vp.cuh"
 
 using namespace dugks;
@@ -37,6 +39,15 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 
 }  // namespace
 
+// tiles of the resident step (dugks_resident.cuh); ntx = 0: the grid does not take it
+struct ResPlan {
+    int ntx = 0, nty = 0, txm = 0, tym = 0, seq = 0, march = 1, threads = 0;
+    size_t smem = 0;
+    uint4* xch = nullptr;       // published cells
+    unsigned* epoch = nullptr;  // steps done per tile, behind them
+    bool owned = false;         // xch is an allocation of its own
+};
+
 struct dugks_ctx {
     int device = 0;
     int nx = 0, ny = 0, precision = 32, kernel = DUGKS_KERNEL_FUSED;
@@ -44,6 +55,7 @@ struct dugks_ctx {
     double bcv[4] = {0, 0, 0, 0};
     double c = 1, dt = 0, lambda = 0, cfl = 0;
     int nc = NC_LARGE;  // equilibrium polynomial coefficients used by the step (3, 4 or 16)
+    int nc_res = NC_LARGE;  // the same for the resident step, which also has 2 (linear equilibria)
     int nc_u = NC_LARGE;  // the same, large enough for b(phi) and int b'^2 of the u-derivative
     double feq_coef[Q][NC_LARGE];
     double a_bp = 0, b_bp = 0, a_tp = 0, b_tp = 0, a_f = 0, b_f = 0, hc = 0;
@@ -72,6 +84,7 @@ struct dugks_ctx {
     bool plain = false;                   // step_vp with the interior variant (long-segment plans)
     int nseg_sp_src = 0;
     SegPlan sp{1, 0, 1};  // step_vp: long segments first, then short ones
+    ResPlan res, res_src;  // the resident step without and with source terms
     long long steps_done = 0;
     // adjoint work buffers (allocated on first use)
     void* adj_ax = nullptr;
@@ -496,6 +509,114 @@ dugks_status plan_fused(dugks_ctx* ctx) {
     return DUGKS_OK;
 }
 
+// cost of a cell, of a face and of the start of a march: warp instructions in FP32, in FP64 the
+// instructions of its slow pipe
+constexpr double kResCost[2][3] = {{120.0, 80.0, 45.0}, {75.0, 75.0, 2.0}};
+constexpr int kResChunk = 1024;  // steps per launch of the resident kernel at most
+
+void* resident_fn(const dugks_ctx* ctx, bool src) {
+    auto pick = [&](auto t) -> void* {
+        using T = decltype(t);
+        switch (ctx->nc_res) {
+            case 2: return src ? (void*)&resident_steps<T, 2, true> : (void*)&resident_steps<T, 2, false>;
+            case 3: return src ? (void*)&resident_steps<T, 3, true> : (void*)&resident_steps<T, 3, false>;
+            case 4: return src ? (void*)&resident_steps<T, 4, true> : (void*)&resident_steps<T, 4, false>;
+            default: return src ? (void*)&resident_steps<T, NC_LARGE, true> : (void*)&resident_steps<T, NC_LARGE, false>;
+        }
+    };
+    return ctx->precision == 32 ? pick(float(0)) : pick(double(0));
+}
+
+void free_resident(ResPlan& r) {
+    if (r.owned) cudaFree(r.xch);
+    r = ResPlan();
+}
+
+// bytes of the published cells (two buffers) and of the step counters behind them; both start at zero
+size_t resident_xch_bytes(const dugks_ctx* ctx, const ResPlan& r) {
+    const size_t words = ctx->precision == 32 ? kResWords<float> : kResWords<double>;
+    return 2 * size_t(r.ntx) * r.nty * size_t(res_slots(r.txm, r.tym)) * words * sizeof(uint4);
+}
+size_t resident_bytes(const dugks_ctx* ctx, const ResPlan& r) {
+    return r.ntx ? resident_xch_bytes(ctx, r) + size_t(r.ntx) * r.nty * sizeof(unsigned) : 0;
+}
+void set_resident_buffers(const dugks_ctx* ctx, ResPlan& r, void* p) {
+    r.xch = static_cast<uint4*>(p);
+    r.epoch = reinterpret_cast<unsigned*>(static_cast<char*>(p) + resident_xch_bytes(ctx, r));
+}
+
+// Tiles of the resident step for nsrc source terms, at most one per SM, and the length of its
+// marches over faces, with the least time per step on one SM: the passes of its warps over cells
+// and over groups of 31 marches, weighed by the instructions of a cell, of a face and of the start
+// of a march.  A grid whose tiles do not fit in shared memory (above about 630^2 cells in FP32 and
+// 435^2 in FP64), or whose tiles are so thin that a CTA has too few threads for their outer
+// neighbours, keeps the row-marching kernels.  Up to that line the resident step was the faster one
+// wherever both were measured (us per step, row-marching against resident): FP32 70x45 20.5 / 1.8,
+// 200^2 with a source term 34 / 3.1, 330x517 16.6 / 4.7, 512^2 18.8 / 6.1, 620^2 20.9 / 8.6;
+// FP64 64^2 150 / 5.9, 200^2 172 / 23, 400^2 155 / 59, 430^2 163 / 70.
+dugks_status plan_resident(dugks_ctx* ctx, int nsrc, ResPlan& r) {
+    free_resident(r);
+    int sms = 0, smem_max = 0, coop = 0;
+    cudaError_t e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device)) != cudaSuccess)
+        return cuda_fail(ctx, e, "cudaDeviceGetAttribute");
+    if (!coop) return DUGKS_OK;
+    void* fn = resident_fn(ctx, nsrc > 0);
+    const size_t room = size_t(smem_max);
+    const int most = ctx->precision == 32 ? kResThreads<float> : kResThreads<double>;
+    auto bytes = [&](int tx, int ty, int seq) {
+        return ctx->precision == 32 ? ResLayout<float>(tx, ty, seq, nsrc).bytes : ResLayout<double>(tx, ty, seq, nsrc).bytes;
+    };
+    const double* cc = kResCost[ctx->precision == 32 ? 0 : 1];
+    double best = INFINITY;
+    ResPlan b;
+    auto tile = [&](int ntx, int& nty, long long& tx, long long& ty) {
+        nty = std::min(ctx->ny, sms / ntx);
+        tx = (ctx->nx + ntx - 1) / ntx;
+        ty = (ctx->ny + nty - 1) / nty;
+        return 2 * (tx + 2) + 2 * ty <= most && tx * ty <= 8192;
+    };
+    int nty;
+    long long tx, ty, fewest = LLONG_MAX;
+    for (int ntx = 1; ntx <= std::min(ctx->nx, sms); ++ntx)
+        if (tile(ntx, nty, tx, ty)) fewest = std::min(fewest, tx * ty);
+    for (int ntx = 1; ntx <= std::min(ctx->nx, sms); ++ntx) {
+        if (!tile(ntx, nty, tx, ty) || tx * ty * 4 > fewest * 5) continue;
+        const int seq = bytes(int(tx), int(ty), 0) <= room ? 0 : 1;
+        if (bytes(int(tx), int(ty), seq) > room) continue;
+        // the threads: one per cell, one lane per face line, one per outer neighbour, as far as they go
+        for (int m = 1; m <= 8; ++m) {
+            const long long gx = ((tx + 1) * ((ty + m - 1) / m) - 2) / 31 + 1, gy = ((ty + 1) * ((tx + m - 1) / m) - 2) / 31 + 1;
+            const long long gc = (tx * ty + 31) / 32, gh = (2 * (tx + 2) + 2 * ty + 31) / 32;
+            const long long nw = std::min<long long>(most / 32, std::max(std::max(seq ? std::max(gx, gy) : gx + gy, gc), gh));
+            // passes of the warps (FP32); in FP64 the pipe of each quarter of the SM takes one warp at a time
+            const long long at_once = ctx->precision == 32 ? nw : 4;
+            const double per = ctx->precision == 32 ? double(std::max<long long>(nw, 4)) / 4.0 : 1.0;
+            auto passes = [&](long long g) { return double((g + at_once - 1) / at_once); };
+            const double faces = seq ? passes(gx) + passes(gy) : passes(gx + gy);
+            const double cost = per * (cc[0] * passes(gc) + faces * (cc[2] + cc[1] * m)) + 0.5 * double(tx + ty);
+            if (cost < best) {
+                best = cost;
+                b.ntx = ntx;
+                b.nty = nty;
+                b.txm = int(tx);
+                b.tym = int(ty);
+                b.seq = seq;
+                b.march = m;
+                b.smem = bytes(int(tx), int(ty), seq);
+                b.threads = int(nw) * 32;
+            }
+        }
+    }
+    if (b.ntx == 0) return DUGKS_OK;
+    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(room))) != cudaSuccess)
+        return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+    r = b;
+    return DUGKS_OK;
+}
+
 // Per-row y metrics of step_vp (rows -1 .. ny at index k + 1) from the y-face and
 // y-cell metrics: the reconstruction weights of the faces below and above each row
 // (Eqs. 2.19, 2.20), its central-difference factor and its flux factor (Eq. 2.12).
@@ -606,6 +727,112 @@ cudaError_t launch_step_any(dugks_ctx* ctx) {
     }
 }
 
+template <typename T, int NC>
+ResConsts<T, NC> make_res_consts(const dugks_ctx* ctx) {
+    const Consts<T, NC> s = make_consts<T, NC>(ctx);
+    ResConsts<T, NC> k;
+    auto v2 = [](T x, T y) {
+        Vec2<T> v;
+        v.x = x;
+        v.y = y;
+        return v;
+    };
+    for (int q = 0; q < 4; ++q)
+        for (int m = 0; m < NC; ++m) {
+            k.hbp[q][m] = v2(s.hbp[PA(q)][m], s.hbp[PB(q)][m]);
+            k.hf[q][m] = v2(s.hf[PA(q)][m], s.hf[PB(q)][m]);
+            k.fq[q][m] = v2(s.feq[PA(q)][m], s.feq[PB(q)][m]);
+        }
+    k.a_bp = s.a_bp;
+    k.b_bp = s.b_bp;
+    k.a_f = s.a_f;
+    k.third = s.third;
+    k.hc = s.hc;
+    for (int w = 0; w < 4; ++w) k.bcv[w] = s.bcv[w];
+    return k;
+}
+
+// n steps of the resident kernel from ctx->cur in place (n <= kResSrcChunk with source terms)
+template <typename T, int NC>
+cudaError_t launch_resident(dugks_ctx* ctx, int n) {
+    const bool src = ctx->nsrc > 0;
+    const ResPlan& r = src ? ctx->res_src : ctx->res;
+    ResArgs<T> a;
+    a.f = static_cast<T*>(ctx->buf[ctx->cur]);
+    a.pitch = ctx->pitch;
+    a.plane = ctx->plane;
+    a.nx = ctx->nx;
+    a.ny = ctx->ny;
+    a.xper = ctx->xper;
+    a.yper = ctx->yper;
+    a.fx = static_cast<const FaceM<T>*>(ctx->fxm);
+    a.fy = static_cast<const FaceM<T>*>(ctx->fym);
+    a.cx = static_cast<const CellM<T>*>(ctx->cxm);
+    a.cy = static_cast<const CellM<T>*>(ctx->cym);
+    a.ntx = r.ntx;
+    a.nty = r.nty;
+    a.txm = r.txm;
+    a.tym = r.tym;
+    a.nsteps = n;
+    a.seq = r.seq;
+    a.march = r.march;
+    a.xch = r.xch;
+    a.epoch = r.epoch;
+    a.err = ctx->err_dev;
+    ResConsts<T, NC> k = make_res_consts<T, NC>(ctx);
+    ResSrc<T> sa{};
+    if (src) {
+        const SrcArgs<T> s = make_src_args<T>(ctx);
+        sa.nterms = s.nterms;
+        sa.first = s.first;
+        for (int q = 0; q < 8; ++q) {
+            sa.dpow[q] = s.dpow[q];
+            sa.db[q] = s.db[q];
+        }
+        for (int i = 0; i < Q; ++i) {
+            sa.kP_g[i] = s.kP_g[i];
+            sa.kP_f[i] = s.kP_f[i];
+            sa.kU_g[i] = s.kU_g[i];
+            sa.kU_f[i] = s.kU_f[i];
+        }
+        if (src_uses_aux(ctx)) {  // pitched planes, the history behind the fields
+            T* aux = static_cast<T*>(ctx->aux[ctx->cur]);
+            sa.field = aux;
+            sa.fplane = ctx->plane;
+            sa.fpitch = sa.hpitch = ctx->pitch;
+            sa.hist = aux + size_t(ctx->nsrc) * ctx->plane;
+        } else {
+            sa.field = s.field;
+            sa.fplane = s.fplane;
+            sa.fpitch = sa.hpitch = ctx->nx;
+            sa.hist = static_cast<T*>(ctx->hist[ctx->cur]);
+        }
+        for (int m = 0; m < n; ++m) {
+            const double t = ctx->tbase + double(ctx->tsteps + m) * ctx->dt;
+            for (int q = 0; q < ctx->nsrc; ++q) {
+                sa.en[m][q] = T(std::exp(ctx->src_rate[q] * t));
+                sa.ep[m][q] = m == 0 && ctx->src_first ? sa.en[m][q] : T(std::exp(ctx->src_rate[q] * (t - ctx->dt)));
+            }
+        }
+    }
+    void* args[] = {&a, &k, &sa};
+    return cudaLaunchCooperativeKernel(resident_fn(ctx, src), dim3(unsigned(r.ntx * r.nty)), dim3(unsigned(r.threads)), args,
+                                       r.smem, ctx->stream);
+}
+
+cudaError_t launch_resident_any(dugks_ctx* ctx, int n) {
+    auto pick = [&](auto t) {
+        using T = decltype(t);
+        switch (ctx->nc_res) {
+            case 2: return launch_resident<T, 2>(ctx, n);
+            case 3: return launch_resident<T, 3>(ctx, n);
+            case 4: return launch_resident<T, 4>(ctx, n);
+            default: return launch_resident<T, NC_LARGE>(ctx, n);
+        }
+    };
+    return ctx->precision == 32 ? pick(float(0)) : pick(double(0));
+}
+
 template <typename T, typename Tin>
 cudaError_t launch_init(dugks_ctx* ctx, const Tin* phi0) {
     const long long n = (long long)ctx->nx * ctx->ny;
@@ -642,6 +869,8 @@ void free_ctx(dugks_ctx* ctx) {
                     static_cast<void*>(ctx->partial), static_cast<void*>(ctx->mass_dev),
                     static_cast<void*>(ctx->err_dev)})
         if (p) cudaFree(p);
+    free_resident(ctx->res);
+    free_resident(ctx->res_src);
     if (prev >= 0) cudaSetDevice(prev);
     delete ctx;
 }
@@ -1132,8 +1361,9 @@ dugks_status dugks_check_feq(const dugks_vset* vset, const dugks_coef* coef, dou
     return margin < 0.0 ? DUGKS_ERR_CONFIG : DUGKS_OK;
 }
 
-dugks_status dugks_create(const dugks_mesh* mesh, const dugks_vset* vset, const dugks_coef* coef, double dt,
-                          const dugks_options* opts, dugks_ctx** out) {
+// stepped_alone: dugks_step will run on it (an instance of a batch only keeps its state there)
+static dugks_status create_ctx(const dugks_mesh* mesh, const dugks_vset* vset, const dugks_coef* coef, double dt,
+                               const dugks_options* opts, bool stepped_alone, dugks_ctx** out) {
     if (!out) return DUGKS_ERR_ARG;
     *out = nullptr;
     dugks_status st = dugks_check_config(mesh, vset, coef, dt);
@@ -1191,6 +1421,7 @@ dugks_status dugks_create(const dugks_mesh* mesh, const dugks_vset* vset, const 
     int maxdeg = 1;
     feq_coefficients(vset, coef, ctx->feq_coef, &maxdeg);
     ctx->nc = maxdeg <= 2 ? 3 : (maxdeg == 3 ? 4 : NC_LARGE);
+    ctx->nc_res = maxdeg <= 1 ? 2 : ctx->nc;
     {  // with u = 0 the step's equilibrium has no b terms, but d feq / d u has b and C/(u u)
         int degb = 0;
         for (int m = 0; m < ctx->nb; ++m)
@@ -1200,23 +1431,33 @@ dugks_status dugks_create(const dugks_mesh* mesh, const dugks_vset* vset, const 
         ctx->nc_u = du <= 2 ? 3 : (du == 3 ? 4 : NC_LARGE);
     }
 
-    const int lane = 128 / int(ctx->elem);  // rows padded to 128 bytes
-    ctx->pitch = ((long long)ctx->nx + lane - 1) / lane * lane;
-    ctx->plane = ctx->pitch * ctx->ny;
-    const size_t bytes = size_t(Q) * size_t(ctx->plane) * ctx->elem;
-
     auto fail = [&](dugks_status s) {
         dugks_status r = s;
         free_ctx(ctx);
         return r;
     };
+    if (stepped_alone && ctx->kernel == DUGKS_KERNEL_FUSED && (st = plan_resident(ctx, 0, ctx->res)) != DUGKS_OK)
+        return fail(st);
+
+    const int lane = 128 / int(ctx->elem);  // rows padded to 128 bytes
+    ctx->pitch = ((long long)ctx->nx + lane - 1) / lane * lane;
+    ctx->plane = ctx->pitch * ctx->ny;
+    const size_t bytes = size_t(Q) * size_t(ctx->plane) * ctx->elem;  // (a multiple of 128)
+
     cudaError_t e;
-    for (int b = 0; b < 2; ++b) {
-        e = cudaMalloc(&ctx->buf[b], bytes);
+    for (int b = 0; b < 2; ++b) {  // the resident step's buffers lie behind the first state buffer
+        size_t n = bytes + (b == 0 ? resident_bytes(ctx, ctx->res) : 0);
+        e = cudaMalloc(&ctx->buf[b], n);
+        if (e == cudaErrorMemoryAllocation && n > bytes) {  // no room for them: row-marching steps
+            cudaGetLastError();
+            ctx->res = ResPlan();
+            e = cudaMalloc(&ctx->buf[b], n = bytes);
+        }
         if (e != cudaSuccess) { cuda_fail(ctx, e, "cudaMalloc(state)"); return fail(DUGKS_ERR_NOMEM); }
-        e = cudaMemsetAsync(ctx->buf[b], 0, bytes, ctx->stream);
+        e = cudaMemsetAsync(ctx->buf[b], 0, n, ctx->stream);
         if (e != cudaSuccess) return fail(cuda_fail(ctx, e, "cudaMemsetAsync"));
     }
+    if (ctx->res.ntx) set_resident_buffers(ctx, ctx->res, static_cast<char*>(ctx->buf[0]) + bytes);
     // metrics
     std::vector<double> dxw, dyw;
     auto upload = [&](void** dst, const void* src, size_t n) -> cudaError_t {
@@ -1277,6 +1518,11 @@ dugks_status dugks_create(const dugks_mesh* mesh, const dugks_vset* vset, const 
     if ((e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) return fail(cuda_fail(ctx, e, "cudaStreamSynchronize"));
     *out = ctx;
     return DUGKS_OK;
+}
+
+dugks_status dugks_create(const dugks_mesh* mesh, const dugks_vset* vset, const dugks_coef* coef, double dt,
+                          const dugks_options* opts, dugks_ctx** out) {
+    return create_ctx(mesh, vset, coef, dt, opts, true, out);
 }
 
 dugks_status dugks_destroy(dugks_ctx* ctx) {
@@ -1340,11 +1586,25 @@ dugks_status dugks_init_phi_host(dugks_ctx* ctx, const double* phi0_host) {
 dugks_status dugks_step(dugks_ctx* ctx, long long n) {
     if (!ctx || n < 0) return DUGKS_ERR_ARG;
     DeviceGuard guard(ctx->device);
-    for (long long s = 0; s < n; ++s) {
-        CK(launch_step_any(ctx));
-        ctx->cur ^= 1;
-        ++ctx->steps_done;
-        ++ctx->tsteps;
+    ResPlan& res = ctx->nsrc > 0 ? ctx->res_src : ctx->res;
+    for (long long s = 0, m; s < n; s += m) {
+        m = 1;
+        if (res.ntx > 0) {  // many steps a launch, the state in place
+            m = std::min<long long>(n - s, ctx->nsrc > 0 ? kResSrcChunk : kResChunk);
+            const cudaError_t e = launch_resident_any(ctx, int(m));
+            if (e == cudaErrorCooperativeLaunchTooLarge) {  // a stream with fewer SMs than the device
+                cudaGetLastError();
+                free_resident(res);
+                m = 0;
+                continue;
+            }
+            CK(e);
+        } else {
+            CK(launch_step_any(ctx));
+            ctx->cur ^= 1;
+        }
+        ctx->steps_done += m;
+        ctx->tsteps += m;
         ctx->t = ctx->tbase + double(ctx->tsteps) * ctx->dt;
         ctx->src_first = false;
     }
@@ -1457,9 +1717,10 @@ dugks_status dugks_info(const dugks_ctx* ctx, dugks_info_t* out) {
     out->dt = ctx->dt;
     out->lambda = ctx->lambda;
     out->cfl = ctx->cfl;
-    out->block_threads = ctx->kernel == DUGKS_KERNEL_NAIVE ? 128 : ctx->nt;
+    const ResPlan& r = ctx->nsrc > 0 ? ctx->res_src : ctx->res;
+    out->block_threads = ctx->kernel == DUGKS_KERNEL_NAIVE ? 128 : (r.ntx > 0 ? r.threads : ctx->nt);
     out->grid_blocks = ctx->kernel == DUGKS_KERNEL_NAIVE ? ((ctx->nx + 127) / 128) * std::min(ctx->ny, 65535)
-                                                         : ctx->nstrips * ctx->nseg;
+                                                         : (r.ntx > 0 ? r.ntx * r.nty : ctx->nstrips * ctx->nseg);
     out->state_bytes = (long long)Q * ctx->plane * (long long)ctx->elem;
     out->time = ctx->t;
     out->nsrc = ctx->nsrc;
@@ -1545,6 +1806,23 @@ dugks_status dugks_set_source(dugks_ctx* ctx, int nterms, const double* rate, co
             CK(cudaMemcpyAsync(static_cast<char*>(ctx->src_field) + size_t(q) * cells * ctx->elem,
                                fields + size_t(order[q]) * cells * ctx->elem, cells * ctx->elem,
                                cudaMemcpyDeviceToDevice, ctx->stream));
+    }
+    if (nterms > 0) {  // (the stream is idle: see above)
+        dugks_status st = plan_resident(ctx, nterms, ctx->res_src);
+        if (st != DUGKS_OK) return st;
+        if (const size_t n = resident_bytes(ctx, ctx->res_src)) {
+            void* p = nullptr;
+            cudaError_t e = cudaMalloc(&p, n);
+            if (e == cudaErrorMemoryAllocation) {  // no room for its buffers: row-marching steps
+                cudaGetLastError();
+                ctx->res_src = ResPlan();
+            } else {
+                CK(e);
+                set_resident_buffers(ctx, ctx->res_src, p);
+                ctx->res_src.owned = true;
+                CK(cudaMemsetAsync(p, 0, n, ctx->stream));
+            }
+        }
     }
     for (int q = 0; q < nterms; ++q) {
         ctx->src_rate[q] = rate[order[q]];
@@ -1705,7 +1983,7 @@ dugks_status dugks_batch_create(int n, const dugks_mesh* meshes, const dugks_vse
     b->ctx.assign(size_t(n), nullptr);
     int nc = 3;
     for (int i = 0; i < n; ++i) {
-        dugks_status st = dugks_create(&meshes[i], &vsets[i], &coefs[i], dts[i], &io, &b->ctx[size_t(i)]);
+        dugks_status st = create_ctx(&meshes[i], &vsets[i], &coefs[i], dts[i], &io, false, &b->ctx[size_t(i)]);
         if (st != DUGKS_OK) return fail(st);
         if (b->ctx[size_t(i)]->nc > 4) return fail(DUGKS_ERR_UNSUPPORTED);  // equilibrium polynomials of degree <= 3
         nc = std::max(nc, b->ctx[size_t(i)]->nc);
