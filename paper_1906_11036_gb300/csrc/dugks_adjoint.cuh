@@ -41,7 +41,8 @@ struct AdjConsts {
 
 template <typename T>
 struct AdjArgs {
-    const T* f;        // forward state ftilde^n, [Q][ny][nx] contiguous
+    const T* f;        // forward state ftilde^n, [Q][ny] rows of nx elements, f_pitch apart
+    long long f_pitch, f_plane;
     const T* mu;       // dJ/d ftilde^{n+1}
     T* lam;            // out: dJ/d ftilde^n
     T* Ax;             // x-face adjoints [Q][ny][nx+1]
@@ -99,19 +100,23 @@ __device__ __forceinline__ T poly_nc(const T (&c)[NC], T x) {
 }
 
 // sum_i w_i d feq_i / d u_a at phi for a = x, y, over the velocities in `mask`
-// (bit i: velocity i), added to du[0], du[1] in double
+// (bit i: velocity i), added to du[0], du[1] in double.  Over all velocities (kAllQ) the rest
+// velocity follows the zeroth moment, its derivative minus the sum of the others: w_i - w_0 weighs
+// the others.  w is nearly the same for all velocities there, and the rounded Au, Bu do not sum to
+// zero, which biased the derivative by up to 1e-5 in FP32.
 template <typename T, int NC>
 __device__ __forceinline__ void add_du(const AdjConsts<T, NC>& ka, T phi, const T (&w)[Q], unsigned mask,
                                        double (&du)[2]) {
     const T bv = poly_nc<T, NC>(ka.bpoly, phi), cv = poly_nc<T, NC>(ka.cpoly, phi);
+    const T w0 = (mask & 1u) ? w[0] : T(0);
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
         T sa = T(0), sb = T(0);
 #pragma unroll
-        for (int i = 0; i < Q; ++i)
+        for (int i = 1; i < Q; ++i)
             if (mask & (1u << i)) {
-                sa = fma(w[i], ka.Au[a][i], sa);
-                sb = fma(w[i], ka.Bu[a][i], sb);
+                sa = fma(w[i] - w0, ka.Au[a][i], sa);
+                sb = fma(w[i] - w0, ka.Bu[a][i], sb);
             }
         du[a] += double(fma(bv, sa, cv * sb));
     }
@@ -178,7 +183,7 @@ __global__ void __launch_bounds__(128) adj_wall_kernel(const StepArgs<T, NC> a, 
         T phi = T(0);
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            ft[i] = g.f[i * cplane + c];
+            ft[i] = g.f[i * g.f_plane + kr * g.f_pitch + j];
             phi += ft[i];
             PG[i] = T(0);
         }
@@ -318,12 +323,12 @@ __global__ void __launch_bounds__(TX * TY) adj_tile_kernel(const StepArgs<T, NC>
 #pragma unroll
             for (int i = 0; i < Q; ++i) P[i] = T(0);  // beyond use, or a corner ghost (zero weights only)
         } else {  // P = fbar^+ (Eq. 2.21) from ftilde, and the mirrored ghost P_g = feq(2 bv - phi) + P - feq(phi)
-            const long long c = (long long)Y.i * nx + X.i;
+            const long long c = Y.i * g.f_pitch + X.i;
             T ft[Q], fe[Q];
             T phi = T(0);
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
-                ft[i] = g.f[i * cplane + c];
+                ft[i] = g.f[i * g.f_plane + c];
                 phi += ft[i];
             }
             feq_all(k, phi, fe);
@@ -527,7 +532,7 @@ __global__ void __launch_bounds__(TX * TY) adj_tile_kernel(const StepArgs<T, NC>
         T phi = T(0);
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            ft[i] = g.f[i * cplane + t];
+            ft[i] = g.f[i * g.f_plane + kr * g.f_pitch + j];
             mu[i] = Mt(i, ty + 1, tx + 1);
             phi += ft[i];
         }

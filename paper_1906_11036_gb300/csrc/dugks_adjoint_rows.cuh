@@ -39,6 +39,8 @@ namespace dugks {
 #define DUGKS_ADJ_ROWS_WALL_MIN_WARPS 12  // the ghost folds need more registers than 16 warps leave
 #endif
 
+static_assert(DUGKS_ADJ_ROWS_MIN_WARPS <= 16 && DUGKS_ADJ_ROWS_WALL_MIN_WARPS <= 16, "the segment plan's row times go to 4 warps");
+
 struct AdjRowLayout {
     static constexpr int WI = 28;                       // owned columns per warp
     static constexpr int BOXW = 36;                     // 32 columns from (xw - 2) rounded down to 16 bytes
@@ -55,10 +57,12 @@ struct AdjConstsP {
     float2 fq[4][NC];           // (feq_PA, feq_PB)
     float2 dq[4][NC];           // (feq_PA', feq_PB') (the top coefficient is zero)
     float2 Au[2][4], Bu[2][4];  // d feq / d u_a = Au b(phi) + Bu Cint(phi) per pair (u of B = u b)
-    float Au0[2], Bu0[2];       // the rest velocity's
     float bpoly[NC], cpoly[NC];
     float a_bp, b_bp, a_tp, b_tp, a_f, b_f;
-    float da_bp, db_bp, da_tp, db_tp, da_f, db_f;  // d/dlambda of the weights
+    // d/dlambda of the weights of f, over b_bp.  Those of feq are the opposite (the weights of each of
+    // Eqs. 2.13, 2.21, 2.22 sum to one), so each enters as da (f - feq), here da / b_bp times
+    // b_bp f - hbp(phi): feq as the forward step rounds it, so the small difference has no bias
+    float da_bp, da_tp, da_f;
     float hc;
     float bcv[4];  // Dirichlet wall values W, E, S, N
 };
@@ -84,14 +88,21 @@ __device__ __forceinline__ F2 ap_dfeq(const AdjConstsP<NC>& k, int q, F2 x) {
     for (int m = NC - 3; m >= 0; --m) s = fma2(s, x, F2{k.dq[q][m]});
     return s;
 }
+// b_bp f - hbp(phi) = b_bp (f - feq) of pair q
+template <int NC>
+__device__ __forceinline__ F2 ap_neq(const AdjConstsP<NC>& k, int q, F2 f, F2 x) {
+    return fma2(f2(k.b_bp), f, f2(-1.f) * ap_hbp(k, q, x));
+}
 __device__ __forceinline__ float hsum(F2 a) { return a.v.x + a.v.y; }
 __device__ __forceinline__ float hdot(F2 a, F2 b) { return fmaf(a.v.x, b.v.x, a.v.y * b.v.y); }
 
 // du[a] += b(phi) sum_q w_q . Au[a][q] + Cint(phi) sum_q w_q . Bu[a][q] over the pairs in
-// qmask (bit q), plus the rest velocity weighted by wz (a row's sum, added in FP64 per row)
+// qmask (bit q).  Over all pairs pass w_q - w_0: the rest velocity follows the zeroth moment, so its
+// derivative is minus the sum of the others, and w is nearly the same for all velocities, which the
+// rounded Au, Bu would not sum to zero (a row's sum, added in FP64 per row)
 template <int NC>
 __device__ __forceinline__ void ap_add_du(const AdjConstsP<NC>& k, float phi, const F2 (&w)[4], unsigned qmask,
-                                          float wz, float (&du)[2]) {
+                                          float (&du)[2]) {
     float bv = k.bpoly[NC - 1], cv = k.cpoly[NC - 1];
 #pragma unroll
     for (int m = NC - 2; m >= 0; --m) {
@@ -107,8 +118,7 @@ __device__ __forceinline__ void ap_add_du(const AdjConstsP<NC>& k, float phi, co
                 sa = fma2(w[q], F2{k.Au[a][q]}, sa);
                 sb = fma2(w[q], F2{k.Bu[a][q]}, sb);
             }
-        const float ta = fmaf(wz, k.Au0[a], hsum(sa)), tb = fmaf(wz, k.Bu0[a], hsum(sb));
-        du[a] += fmaf(bv, ta, cv * tb);
+        du[a] += fmaf(bv, hsum(sa), cv * hsum(sb));
     }
 }
 
@@ -139,31 +149,32 @@ __device__ __forceinline__ void ap_ghost_fold(const AdjConstsP<NC>& k, const V9&
     const float phc = vsum(ft), phg = 2.f * bv - phc;
     const F2 xc = f2(phc), xg = f2(phg);
     const F2 c1 = f2(k.b_bp - 1.f);
-    F2 pb = f2(0.f), dcs = f2(0.f), dgs = f2(0.f), fcs = f2(0.f), sp = f2(0.f);
+    F2 pb = f2(0.f), dcs = f2(0.f), dgs = f2(0.f), ncs = f2(0.f), sp = f2(0.f);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const F2 dc = ap_dfeq(k, q, xc), dg = ap_dfeq(k, q, xg), fc = ap_feq(k, q, xc);
+        const F2 dc = ap_dfeq(k, q, xc), dg = ap_dfeq(k, q, xg), nc = ap_neq(k, q, ft.p[q], xc);
         pb = fma2(B.p[q], fma2(c1, dc, f2(-1.f) * dg), pb);
         dcs = dcs + dc;
         dgs = dgs + dg;
-        fcs = fcs + fc;
-        sp = fma2(B.p[q], fma2(f2(k.da_bp), ft.p[q], f2(k.db_bp) * fc), sp);
+        ncs = ncs + nc;
+        sp = fma2(B.p[q], nc, sp);
     }
     // the rest velocity's derivatives and equilibrium follow the zeroth moment
-    const float dc0 = 1.f - hsum(dcs), dg0 = 1.f - hsum(dgs), fc0 = phc - hsum(fcs);
+    const float dc0 = 1.f - hsum(dcs), dg0 = 1.f - hsum(dgs), nc0 = -hsum(ncs);
     const float phibar = fmaf(B.z, fmaf(k.b_bp - 1.f, dc0, -dg0), hsum(pb));
     const F2 ph2 = f2(phibar);
 #pragma unroll
     for (int q = 0; q < 4; ++q) v.p[q] = fma2(f2(k.a_bp), B.p[q], ph2);
     v.z = fmaf(k.a_bp, B.z, phibar);
-    rl += hsum(sp) + B.z * fmaf(k.da_bp, ft.z, k.db_bp * fc0);
+    rl = fmaf(k.da_bp, fmaf(B.z, nc0, hsum(sp)), rl);
     if (WU) {  // (b_bp - 1) feq(phi_c) and feq(phi_g) in P_g
         F2 w[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) w[q] = c1 * B.p[q];
-        ap_add_du(k, phc, w, 0xFu, (k.b_bp - 1.f) * B.z, ru);
-        F2 wg[4] = {B.p[0], B.p[1], B.p[2], B.p[3]};
-        ap_add_du(k, phg, wg, 0xFu, B.z, ru);
+        for (int q = 0; q < 4; ++q) w[q] = B.p[q] - f2(B.z);
+        ap_add_du(k, phg, w, 0xFu, ru);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w[q] = c1 * w[q];
+        ap_add_du(k, phc, w, 0xFu, ru);
     }
 }
 
@@ -241,10 +252,11 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
 #pragma unroll
             for (int q = 0; q < 4; ++q) v.p[q] = f2(0.f);
         } else {
-            const float* src = (which ? g.mu : g.f) + (long long)(which ? wrow(r) : frow(r)) * nx + jw;
+            const float* src = which ? g.mu + (long long)wrow(r) * nx + jw : g.f + frow(r) * g.f_pitch + jw;
+            const long long pl = which ? cplane : g.f_plane;
             v.z = src[0];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) v.p[q] = f2(src[PA(q) * cplane], src[PB(q) * cplane]);
+            for (int q = 0; q < 4; ++q) v.p[q] = f2(src[PA(q) * pl], src[PB(q) * pl]);
         }
     };
 
@@ -345,20 +357,19 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
 #pragma unroll
             for (int s = 0; s < 3; ++s) {
                 const int q = s == 0 ? 0 : s + 1;
-                const F2 fe = ap_feq(k, q, pb2);
                 sgp = fma2(gv[s], ap_dfeq(k, q, pb2), sgp);
-                sdp = fma2(gv[s], fma2(f2(k.da_f), fb[s], f2(k.db_f) * fe), sdp);
+                sdp = fma2(gv[s], ap_neq(k, q, fb[s], pb2), sdp);
             }
             const float sg = hsum(sgp), bsg = k.b_f * sg;
             // (with an x-wall the ghost lane j = -1 counts the wall face west of column 0)
             if ((owner || (XW && j == -1)) && n - 1 >= y0 && n - 1 < y1) {
-                rl += hsum(sdp);
+                rl = fmaf(k.da_f, hsum(sdp), rl);
                 if (WU) {  // Eq. 2.22: b_f feq(phi_b) of the crossing velocities
                     F2 w[4];
                     w[1] = f2(0.f);
 #pragma unroll
                     for (int s = 0; s < 3; ++s) w[s == 0 ? 0 : s + 1] = f2(k.b_f) * gv[s];
-                    ap_add_du(k, phib, w, 0xDu, 0.f, ru);
+                    ap_add_du(k, phib, w, 0xDu, ru);
                 }
             }
             // the face's A at its right cell (the lane to the east)
@@ -417,22 +428,21 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
             F2 sgp = f2(0.f), sdp = f2(0.f);
 #pragma unroll
             for (int s = 0; s < 3; ++s) {
-                const F2 fe = ap_feq(k, s + 1, pb2);
                 sgp = fma2(gv[s], ap_dfeq(k, s + 1, pb2), sgp);
-                sdp = fma2(gv[s], fma2(f2(k.da_f), fb[s], f2(k.db_f) * fe), sdp);
+                sdp = fma2(gv[s], ap_neq(k, s + 1, fb[s], pb2), sdp);
             }
             const float bsg = k.b_f * hsum(sgp);
             F2 A[3];
 #pragma unroll
             for (int s = 0; s < 3; ++s) A[s] = fma2(f2(k.a_f), gv[s], f2(bsg));
             if (owner && (n < y1 || (YW && n == ny))) {  // (a y-wall's top face is its own face)
-                rl += hsum(sdp);
+                rl = fmaf(k.da_f, hsum(sdp), rl);
                 if (WU) {
                     F2 w[4];
                     w[0] = f2(0.f);
 #pragma unroll
                     for (int s = 0; s < 3; ++s) w[s + 1] = f2(k.b_f) * gv[s];
-                    ap_add_du(k, phib, w, 0xEu, 0.f, ru);
+                    ap_add_du(k, phib, w, 0xEu, ru);
                 }
             }
             // normal weights into rows n - 1 (below) and n (above); pair 0 and the rest velocity
@@ -490,18 +500,17 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
             const float phi = vsum(ft);
             const F2 x2 = f2(phi);
             F2 w[4];
-            F2 pb = f2(0.f), dsum = f2(0.f), fsum = f2(0.f), sp = f2(0.f);
+            F2 pb = f2(0.f), dsum = f2(0.f), nsum = f2(0.f), sp = f2(0.f);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const F2 de = ap_dfeq(k, q, x2), fe = ap_feq(k, q, x2);
+                const F2 de = ap_dfeq(k, q, x2), ne = ap_neq(k, q, ft.p[q], x2);
                 w[q] = fma2(f2(k.b_bp), Ba.p[q], f2(k.b_tp) * mu.p[q]);
                 pb = fma2(w[q], de, pb);
                 dsum = dsum + de;
-                fsum = fsum + fe;
-                sp = fma2(Ba.p[q], fma2(f2(k.da_bp), ft.p[q], f2(k.db_bp) * fe), sp);
-                sp = fma2(mu.p[q], fma2(f2(k.da_tp), ft.p[q], f2(k.db_tp) * fe), sp);
+                nsum = nsum + ne;
+                sp = fma2(fma2(f2(k.da_bp), Ba.p[q], f2(k.da_tp) * mu.p[q]), ne, sp);
             }
-            const float de0 = 1.f - hsum(dsum), fe0 = phi - hsum(fsum);  // rest velocity: zeroth moment
+            const float de0 = 1.f - hsum(dsum), ne0 = -hsum(nsum);  // rest velocity: zeroth moment
             const float wz = fmaf(k.b_bp, Ba.z, k.b_tp * mu.z);
             const float phibar = fmaf(wz, de0, hsum(pb));
             V9 addv;  // folds of the mirrored ghosts of this cell (walls)
@@ -546,8 +555,12 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
                 }
             }
             if (owner) {
-                rl += hsum(sp) + fmaf(Ba.z, fmaf(k.da_bp, ft.z, k.db_bp * fe0), mu.z * fmaf(k.da_tp, ft.z, k.db_tp * fe0));
-                if (WU) ap_add_du(k, phi, w, 0xFu, wz, ru);  // b_bp feq(phi) in P, b_tp feq(phi) in ftilde^+
+                rl += fmaf(fmaf(k.da_bp, Ba.z, k.da_tp * mu.z), ne0, hsum(sp));
+                if (WU) {  // b_bp feq(phi) in P, b_tp feq(phi) in ftilde^+
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) w[q] = w[q] - f2(wz);
+                    ap_add_du(k, phi, w, 0xFu, ru);
+                }
                 if constexpr (WALL) {
                     rl += addl;
                     if (WU) {

@@ -50,6 +50,7 @@ struct ResPlan {
 
 struct dugks_ctx {
     int device = 0;
+    int sms = 1;  // SMs of the device
     int nx = 0, ny = 0, precision = 32, kernel = DUGKS_KERNEL_FUSED;
     int xper = 1, yper = 1;
     double bcv[4] = {0, 0, 0, 0};
@@ -395,19 +396,18 @@ EncodeTiledFn tiled_encoder(dugks_ctx* ctx) {
     return encode;
 }
 
-dugks_status make_tensor_maps(dugks_ctx* ctx) {
+// TMA descriptors of n states laid out like the context's own buffers
+dugks_status make_state_maps(dugks_ctx* ctx, void* const* base, int n, CUtensorMap* out) {
     EncodeTiledFn encode = tiled_encoder(ctx);
     if (!encode) return DUGKS_ERR_CUDA;
-    const int align = 16 / int(ctx->elem);
     const cuuint64_t dims[3] = {cuuint64_t(ctx->nx), cuuint64_t(ctx->ny), cuuint64_t(Q)};
     const cuuint64_t strides[2] = {cuuint64_t(ctx->pitch) * ctx->elem, cuuint64_t(ctx->plane) * ctx->elem};
     const cuuint32_t box[3] = {cuuint32_t(ctx->precision == 32 ? WarpLayout<float>::BOXW : WarpLayout<double>::BOXW),
                                1u, cuuint32_t(Q)};
-    (void)align;
     const cuuint32_t estr[3] = {1u, 1u, 1u};
-    for (int b = 0; b < 2; ++b) {
-        CUresult r = encode(&ctx->tmap[b], ctx->precision == 32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64,
-                            3, ctx->buf[b], dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    for (int b = 0; b < n; ++b) {
+        CUresult r = encode(&out[b], ctx->precision == 32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64,
+                            3, base[b], dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) {
@@ -677,18 +677,28 @@ SrcArgs<T> make_src_args(const dugks_ctx* ctx) {
     return sa;
 }
 
+// one step reads `in` (descriptor map) and writes `out`, both laid out like the context's buffers
+struct StepIO {
+    const void* in;
+    void* out;
+    const CUtensorMap* map;
+};
+StepIO own_io(const dugks_ctx* ctx) { return {ctx->buf[ctx->cur], ctx->buf[ctx->cur ^ 1], &ctx->tmap[ctx->cur]}; }
+
 template <typename T, int NC>
-cudaError_t launch_step(dugks_ctx* ctx) {
-    const StepArgs<T, NC> a = make_args<T, NC>(ctx, ctx->cur);
+cudaError_t launch_step(dugks_ctx* ctx, const StepIO& io) {
+    StepArgs<T, NC> a = make_args<T, NC>(ctx, ctx->cur);
+    a.fin = static_cast<const T*>(io.in);
+    a.fout = static_cast<T*>(io.out);
     const Consts<T, NC> k = make_consts<T, NC>(ctx);
     if (ctx->nsrc > 0) {  // the fused kernel with the source terms: velocity pairs in FP32, else scalar
         dim3 grid(ctx->nstrips, ctx->nseg_src);
         if constexpr (sizeof(T) == 4 && NC != NC_LARGE)
             step_vp_src<NC><<<dim3(ctx->nstrips, ctx->nseg_sp_src), 32, src_vp_smem(ctx), ctx->stream>>>(
-                ctx->tmap[ctx->cur], a, make_constsp<NC>(ctx), ctx->rowy, ctx->sp_src, ctx->stages,
+                *io.map, a, make_constsp<NC>(ctx), ctx->rowy, ctx->sp_src, ctx->stages,
                 make_src_args<float>(ctx), ctx->taux[ctx->cur]);
         else
-            fused_step_src<T, NC><<<grid, 32, fused_smem(ctx), ctx->stream>>>(ctx->tmap[ctx->cur], a, k,
+            fused_step_src<T, NC><<<grid, 32, fused_smem(ctx), ctx->stream>>>(*io.map, a, k,
                                                                              ctx->seg_rows_src, ctx->stages,
                                                                              make_src_args<T>(ctx));
         return cudaGetLastError();
@@ -701,29 +711,29 @@ cudaError_t launch_step(dugks_ctx* ctx) {
         if constexpr (sizeof(T) == 4 && NC != NC_LARGE)
             if (ctx->plain)
                 step_vp<NC, true><<<grid, 32, fused_smem(ctx), ctx->stream>>>(
-                    ctx->tmap[ctx->cur], a, make_constsp<NC>(ctx), ctx->rowy, ctx->sp, ctx->stages);
+                    *io.map, a, make_constsp<NC>(ctx), ctx->rowy, ctx->sp, ctx->stages);
             else
                 step_vp<NC, false><<<grid, 32, fused_smem(ctx), ctx->stream>>>(
-                    ctx->tmap[ctx->cur], a, make_constsp<NC>(ctx), ctx->rowy, ctx->sp, ctx->stages);
+                    *io.map, a, make_constsp<NC>(ctx), ctx->rowy, ctx->sp, ctx->stages);
         else
-            fused_step<T, NC><<<grid, 32, fused_smem(ctx), ctx->stream>>>(ctx->tmap[ctx->cur], a, k, ctx->seg_rows,
+            fused_step<T, NC><<<grid, 32, fused_smem(ctx), ctx->stream>>>(*io.map, a, k, ctx->seg_rows,
                                                                          ctx->stages);
     }
     return cudaGetLastError();
 }
 
-cudaError_t launch_step_any(dugks_ctx* ctx) {
+cudaError_t launch_step_any(dugks_ctx* ctx, const StepIO& io) {
     if (ctx->precision == 32) {
         switch (ctx->nc) {
-            case 3: return launch_step<float, 3>(ctx);
-            case 4: return launch_step<float, 4>(ctx);
-            default: return launch_step<float, NC_LARGE>(ctx);
+            case 3: return launch_step<float, 3>(ctx, io);
+            case 4: return launch_step<float, 4>(ctx, io);
+            default: return launch_step<float, NC_LARGE>(ctx, io);
         }
     }
     switch (ctx->nc) {
-        case 3: return launch_step<double, 3>(ctx);
-        case 4: return launch_step<double, 4>(ctx);
-        default: return launch_step<double, NC_LARGE>(ctx);
+        case 3: return launch_step<double, 3>(ctx, io);
+        case 4: return launch_step<double, 4>(ctx, io);
+        default: return launch_step<double, NC_LARGE>(ctx, io);
     }
 }
 
@@ -752,13 +762,17 @@ ResConsts<T, NC> make_res_consts(const dugks_ctx* ctx) {
     return k;
 }
 
-// n steps of the resident kernel from ctx->cur in place (n <= kResSrcChunk with source terms)
+// n steps of the resident kernel (n <= kResSrcChunk with source terms) from `in` to `out` (the same
+// buffer, or not); rec: also keep the states after steps 1 .. n - 1, one state's bytes apart
 template <typename T, int NC>
-cudaError_t launch_resident(dugks_ctx* ctx, int n) {
+cudaError_t launch_resident(dugks_ctx* ctx, int n, const void* in, void* out, void* rec) {
     const bool src = ctx->nsrc > 0;
     const ResPlan& r = src ? ctx->res_src : ctx->res;
     ResArgs<T> a;
-    a.f = static_cast<T*>(ctx->buf[ctx->cur]);
+    a.fin = static_cast<const T*>(in);
+    a.fout = static_cast<T*>(out);
+    a.rec = static_cast<T*>(rec);
+    a.rstride = (long long)Q * ctx->plane;
     a.pitch = ctx->pitch;
     a.plane = ctx->plane;
     a.nx = ctx->nx;
@@ -820,17 +834,34 @@ cudaError_t launch_resident(dugks_ctx* ctx, int n) {
                                        r.smem, ctx->stream);
 }
 
-cudaError_t launch_resident_any(dugks_ctx* ctx, int n) {
+cudaError_t launch_resident_any(dugks_ctx* ctx, int n, const void* in, void* out, void* rec) {
     auto pick = [&](auto t) {
         using T = decltype(t);
         switch (ctx->nc_res) {
-            case 2: return launch_resident<T, 2>(ctx, n);
-            case 3: return launch_resident<T, 3>(ctx, n);
-            case 4: return launch_resident<T, 4>(ctx, n);
-            default: return launch_resident<T, NC_LARGE>(ctx, n);
+            case 2: return launch_resident<T, 2>(ctx, n, in, out, rec);
+            case 3: return launch_resident<T, 3>(ctx, n, in, out, rec);
+            case 4: return launch_resident<T, 4>(ctx, n, in, out, rec);
+            default: return launch_resident<T, NC_LARGE>(ctx, n, in, out, rec);
         }
     };
     return ctx->precision == 32 ? pick(float(0)) : pick(double(0));
+}
+
+// steps a resident launch may take (0: the grid runs the row-marching kernels)
+long long resident_chunk(const dugks_ctx* ctx) {
+    if ((ctx->nsrc > 0 ? ctx->res_src : ctx->res).ntx == 0) return 0;
+    return ctx->nsrc > 0 ? kResSrcChunk : kResChunk;
+}
+
+// launch_resident_any; cudaErrorCooperativeLaunchTooLarge (a stream with fewer SMs than the device)
+// leaves the context on the row-marching kernels and the state as it was
+cudaError_t run_resident(dugks_ctx* ctx, int n, const void* in, void* out, void* rec) {
+    const cudaError_t e = launch_resident_any(ctx, n, in, out, rec);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        (ctx->nsrc > 0 ? ctx->res_src : ctx->res).ntx = 0;
+    }
+    return e;
 }
 
 template <typename T, typename Tin>
@@ -941,17 +972,13 @@ AdjConstsP<NC> make_adj_consts_p(const dugks_ctx* ctx) {
             p.Bu[ax][q] = make_float2(ka.Bu[ax][PA(q)], ka.Bu[ax][PB(q)]);
         }
     }
-    for (int ax = 0; ax < 2; ++ax) {
-        p.Au0[ax] = ka.Au[ax][0];
-        p.Bu0[ax] = ka.Bu[ax][0];
-    }
     for (int m = 0; m < NC; ++m) {
         p.bpoly[m] = ka.bpoly[m];
         p.cpoly[m] = ka.cpoly[m];
     }
-    p.a_bp = ka.a_bp; p.b_bp = ka.b_bp; p.a_tp = ka.a_tp; p.b_tp = ka.b_tp; p.a_f = ka.a_f; p.b_f = ka.b_f;
-    p.da_bp = ka.da_bp; p.db_bp = ka.db_bp; p.da_tp = ka.da_tp; p.db_tp = ka.db_tp;
-    p.da_f = ka.da_f; p.db_f = ka.db_f;
+    p.a_bp = k.a_bp; p.b_bp = k.b_bp; p.a_tp = k.a_tp; p.b_tp = k.b_tp; p.a_f = k.a_f; p.b_f = k.b_f;  // the forward step's
+    p.da_bp = float(double(ka.da_bp) / k.b_bp); p.da_tp = float(double(ka.da_tp) / k.b_bp);
+    p.da_f = float(double(ka.da_f) / k.b_bp);
     p.hc = k.hc;
     for (int w = 0; w < 4; ++w) p.bcv[w] = k.bcv[w];
     return p;
@@ -977,7 +1004,40 @@ long long adj_wall_cells(const dugks_ctx* ctx) {
     return nrc + ncc;
 }
 int adj_wall_blocks(const dugks_ctx* ctx) { return int((adj_wall_cells(ctx) + kAdjThreads - 1) / kAdjThreads); }
-int adj_partials(const dugks_ctx* ctx) { return adj_tile_blocks(ctx) + adj_wall_blocks(ctx); }
+
+// The row-marching FP32 adjoint (adj_rows_kernel): strips and row segments, one partial per warp.
+// A segment passes four rows more than it owns.  Grids of several waves take 16-row segments
+// (2048^2: 180 us against 186 with 24 rows and 200 with 29).  Below two waves the segment length
+// minimises the time: rows passed times the time of a row with so many warps on a quarter of an SM
+// (measured: 1.95, 2.07, 2.4, 2.84 us for 1 .. 4 warps), a launch of more than a wave with about a
+// third of one more for its tail.  512^2: 22.7 us with 4-row segments (4 warps) against 24.8 with 8
+// (2 warps), 26.8 with 6 (3 warps) and 39 with 16; with walls (3 warps at most) 22.7 us with 8.
+constexpr int kAdjRowSeg = 16;
+void adj_row_plan(const dugks_ctx* ctx, int& strips, int& seg, int& nseg) {
+    strips = (ctx->nx + AdjRowLayout::WI - 1) / AdjRowLayout::WI;
+    static const double row_us[4] = {1.95, 2.07, 2.4, 2.84};
+    const int per = (ctx->xper && ctx->yper ? DUGKS_ADJ_ROWS_MIN_WARPS : DUGKS_ADJ_ROWS_WALL_MIN_WARPS) / 4;
+    auto waves = [&](int s) { return double(strips) * ((ctx->ny + s - 1) / s) / (4.0 * per * ctx->sms); };
+    seg = kAdjRowSeg;
+    if (waves(kAdjRowSeg) <= 2.0) {
+        double best = INFINITY;
+        for (int s = 4; s <= 24; ++s) {
+            const double w = waves(s);
+            const double t = w <= 1.0 ? row_us[std::max(0, int(std::ceil(w * per)) - 1)] : (w + 0.35) * row_us[per - 1];
+            if (w <= 2.0 && t * (s + 4) < best) {
+                best = t * (s + 4);
+                seg = s;
+            }
+        }
+    }
+    seg = std::min(seg, ctx->ny);
+    nseg = (ctx->ny + seg - 1) / seg;
+}
+int adj_partials(const dugks_ctx* ctx) {
+    int strips, seg, nseg;
+    adj_row_plan(ctx, strips, seg, nseg);
+    return std::max(adj_tile_blocks(ctx) + adj_wall_blocks(ctx), strips * nseg);
+}
 // blocks of init_adjoint_kernel
 int init_blocks(const dugks_ctx* ctx) {
     return int(std::min<long long>(((long long)ctx->nx * ctx->ny + 255) / 256, 65535));
@@ -1014,19 +1074,8 @@ cudaError_t launch_adj_sum(dugks_ctx* ctx, double* dj_dalpha, double* dj_du) {
 #define DUGKS_ADJ_ROW_STAGES 4
 #endif
 constexpr int kAdjRowStages = DUGKS_ADJ_ROW_STAGES;  // row stages in flight per warp (>= 3)
-// Segments: as many as the 16-row minimum allows up to 96 warps per SM over the launch.  Short
-// segments even out the end of the launch: 2048^2 took 186 us with 16-row segments against
-// 200 us with 29-row ones (36 warps per SM) and 215 us with 24 warps per SM.
-#ifndef DUGKS_ADJ_ROW_WARPS_PER_SM
-#define DUGKS_ADJ_ROW_WARPS_PER_SM 96
-#endif
-#ifndef DUGKS_ADJ_ROW_MIN_SEG
-#define DUGKS_ADJ_ROW_MIN_SEG 16
-#endif
-constexpr int kAdjRowWarpsPerSM = DUGKS_ADJ_ROW_WARPS_PER_SM;  // warps per SM over one launch (segment count)
-constexpr int kAdjRowMinSeg = DUGKS_ADJ_ROW_MIN_SEG;           // rows per segment at least
-// It is used from 1 M cells up (2048^2: 243 us against 506 us for the tiled kernel, 1024^2:
-// 91 against 144 us; on 512^2, with too few warps in flight, the tiled kernel is faster), or
+// It is used where its segments give every SM six warps (512^2 periodic: 22.7 us against 37.1 us
+// for the tiled kernel, with walls 22.7 against 44.1; 256^2, below the line: 16.6 against 14.6), or
 // wherever it applies when dugks_set_adjoint_kernel asked for it.
 bool adj_rows_ok(const dugks_ctx* ctx, const void* f, const void* mu) {
     const bool applies = ctx->precision == 32 && ctx->nc != NC_LARGE && ctx->nx % 4 == 0 &&
@@ -1034,7 +1083,9 @@ bool adj_rows_ok(const dugks_ctx* ctx, const void* f, const void* mu) {
                          (reinterpret_cast<uintptr_t>(mu) % 16) == 0;
     if (!applies || ctx->adj_kernel == DUGKS_ADJ_TILED) return false;
     if (ctx->adj_kernel == DUGKS_ADJ_ROWS) return true;
-    return (long long)ctx->nx * ctx->ny >= 1024LL * 1024;
+    int strips, seg, nseg;
+    adj_row_plan(ctx, strips, seg, nseg);
+    return (long long)strips * nseg >= 6LL * ctx->sms;
 }
 
 template <int NC>
@@ -1045,29 +1096,19 @@ cudaError_t launch_adjoint_rows(dugks_ctx* ctx, const StepArgs<float, NC>& a, co
     using L = AdjRowLayout;
     CUtensorMap tm[2];
     const cuuint64_t dims[3] = {cuuint64_t(ctx->nx), cuuint64_t(ctx->ny), cuuint64_t(Q)};
-    const cuuint64_t strides[2] = {cuuint64_t(ctx->nx) * 4, cuuint64_t(ctx->nx) * ctx->ny * 4};
+    const cuuint64_t strides[2][2] = {{cuuint64_t(g.f_pitch) * 4, cuuint64_t(g.f_plane) * 4},
+                                      {cuuint64_t(ctx->nx) * 4, cuuint64_t(ctx->nx) * ctx->ny * 4}};
     const cuuint32_t box[3] = {cuuint32_t(L::BOXW), 1u, cuuint32_t(Q)};
     const cuuint32_t estr[3] = {1u, 1u, 1u};
     const void* base[2] = {f, mu};
     for (int b = 0; b < 2; ++b)
-        if (encode(&tm[b], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base[b]), dims, strides, box, estr,
+        if (encode(&tm[b], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base[b]), dims, strides[b], box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
-    int sms = 0;
-    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
-    if (e != cudaSuccess) return e;
-    // about kAdjRowWarpsPerSM warps per SM over the launch, segments of at least kAdjRowMinSeg
-    // rows, one partial per warp
-    const int strips = (ctx->nx + L::WI - 1) / L::WI;
-    const long long cap = adj_partials(ctx);
-    long long nseg = std::max<long long>(1, (long long)kAdjRowWarpsPerSM * sms / strips);
-    nseg = std::min<long long>(nseg, std::max(1, ctx->ny / kAdjRowMinSeg));
-    nseg = std::max<long long>(1, std::min<long long>(nseg, cap / strips));
-    const int seg = int((ctx->ny + nseg - 1) / nseg);
-    nseg = (ctx->ny + seg - 1) / seg;
-    if ((long long)strips * nseg > cap) return cudaErrorInvalidConfiguration;
-    ctx->adj_used = int(strips * nseg);  // the sums read the slots this launch writes
+    int strips, seg, nseg;
+    adj_row_plan(ctx, strips, seg, nseg);
+    ctx->adj_used = strips * nseg;  // the sums read the slots this launch writes
     const AdjConstsP<NC> kp = make_adj_consts_p<NC>(ctx);
     const dim3 grid(strips, unsigned(nseg));
     const size_t smem = L::bytes(kAdjRowStages);
@@ -1090,8 +1131,8 @@ cudaError_t launch_adjoint_rows(dugks_ctx* ctx, const StepArgs<float, NC>& a, co
 // dj_dalpha set, are summed into *dj_dalpha (and dj_du[0..1] if set).  want_u: also form
 // the u-derivative.
 template <typename T, int NC>
-cudaError_t launch_adjoint_step(dugks_ctx* ctx, const void* f, const void* mu, void* lam, double* dj_dalpha,
-                                double* dj_du, bool want_u, bool accumulate) {
+cudaError_t launch_adjoint_step(dugks_ctx* ctx, const void* f, long long f_pitch, const void* mu, void* lam,
+                                double* dj_dalpha, double* dj_du, bool want_u, bool accumulate) {
     StepArgs<T, NC> a = make_args<T, NC>(ctx, 0);
     a.fin = static_cast<const T*>(f);  // the adjoint reads contiguous [Q][ny][nx] states
     a.pitch = ctx->nx;
@@ -1100,6 +1141,8 @@ cudaError_t launch_adjoint_step(dugks_ctx* ctx, const void* f, const void* mu, v
     const AdjConsts<T, NC> ka = make_adj_consts<T, NC>(ctx);
     AdjArgs<T> g;
     g.f = static_cast<const T*>(f);
+    g.f_pitch = f_pitch;
+    g.f_plane = f_pitch * ctx->ny;
     g.mu = static_cast<const T*>(mu);
     g.lam = static_cast<T*>(lam);
     g.Ax = static_cast<T*>(ctx->adj_ax);
@@ -1130,20 +1173,21 @@ cudaError_t launch_adjoint_step(dugks_ctx* ctx, const void* f, const void* mu, v
     return cudaGetLastError();
 }
 
-cudaError_t launch_adjoint_step_any(dugks_ctx* ctx, const void* f, const void* mu, void* lam, double* dj_dalpha,
-                                    double* dj_du, bool want_u, bool accumulate) {
+// f: rows f_pitch elements apart (nx: contiguous, or the pitch of the context's own states)
+cudaError_t launch_adjoint_step_any(dugks_ctx* ctx, const void* f, long long f_pitch, const void* mu, void* lam,
+                                    double* dj_dalpha, double* dj_du, bool want_u, bool accumulate) {
     const int nc = want_u ? std::max(ctx->nc, ctx->nc_u) : ctx->nc;
     if (ctx->precision == 32) {
         switch (nc) {
-            case 3: return launch_adjoint_step<float, 3>(ctx, f, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
-            case 4: return launch_adjoint_step<float, 4>(ctx, f, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
-            default: return launch_adjoint_step<float, NC_LARGE>(ctx, f, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
+            case 3: return launch_adjoint_step<float, 3>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
+            case 4: return launch_adjoint_step<float, 4>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
+            default: return launch_adjoint_step<float, NC_LARGE>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
         }
     }
     switch (nc) {
-        case 3: return launch_adjoint_step<double, 3>(ctx, f, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
-        case 4: return launch_adjoint_step<double, 4>(ctx, f, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
-        default: return launch_adjoint_step<double, NC_LARGE>(ctx, f, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
+        case 3: return launch_adjoint_step<double, 3>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
+        case 4: return launch_adjoint_step<double, 4>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
+        default: return launch_adjoint_step<double, NC_LARGE>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
     }
 }
 
@@ -1382,6 +1426,10 @@ static dugks_status create_ctx(const dugks_mesh* mesh, const dugks_vset* vset, c
         ctx->device = o.device;
     }
     DeviceGuard guard(ctx->device);
+    if (cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) {
+        delete ctx;
+        return DUGKS_ERR_CUDA;
+    }
     ctx->nx = mesh->nx;
     ctx->ny = mesh->ny;
     ctx->precision = o.precision;
@@ -1512,7 +1560,7 @@ static dugks_status create_ctx(const dugks_mesh* mesh, const dugks_vset* vset, c
     if (ctx->kernel == DUGKS_KERNEL_FUSED) {
         st = plan_fused(ctx);
         if (st != DUGKS_OK) return fail(st);
-        st = make_tensor_maps(ctx);
+        st = make_state_maps(ctx, ctx->buf, 2, ctx->tmap);
         if (st != DUGKS_OK) return fail(st);
     }
     if ((e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) return fail(cuda_fail(ctx, e, "cudaStreamSynchronize"));
@@ -1586,21 +1634,18 @@ dugks_status dugks_init_phi_host(dugks_ctx* ctx, const double* phi0_host) {
 dugks_status dugks_step(dugks_ctx* ctx, long long n) {
     if (!ctx || n < 0) return DUGKS_ERR_ARG;
     DeviceGuard guard(ctx->device);
-    ResPlan& res = ctx->nsrc > 0 ? ctx->res_src : ctx->res;
     for (long long s = 0, m; s < n; s += m) {
-        m = 1;
-        if (res.ntx > 0) {  // many steps a launch, the state in place
-            m = std::min<long long>(n - s, ctx->nsrc > 0 ? kResSrcChunk : kResChunk);
-            const cudaError_t e = launch_resident_any(ctx, int(m));
-            if (e == cudaErrorCooperativeLaunchTooLarge) {  // a stream with fewer SMs than the device
-                cudaGetLastError();
-                free_resident(res);
+        m = std::min<long long>(n - s, resident_chunk(ctx));
+        if (m > 0) {  // many steps a launch, the state in place
+            const cudaError_t e = run_resident(ctx, int(m), ctx->buf[ctx->cur], ctx->buf[ctx->cur], nullptr);
+            if (e == cudaErrorCooperativeLaunchTooLarge) {
                 m = 0;
                 continue;
             }
             CK(e);
         } else {
-            CK(launch_step_any(ctx));
+            m = 1;
+            CK(launch_step_any(ctx, own_io(ctx)));
             ctx->cur ^= 1;
         }
         ctx->steps_done += m;
@@ -1845,7 +1890,7 @@ dugks_status dugks_adjoint_step(dugks_ctx* ctx, const void* f_dev, const void* m
     DeviceGuard guard(ctx->device);
     dugks_status st = adj_alloc(ctx);
     if (st != DUGKS_OK) return st;
-    CK(launch_adjoint_step_any(ctx, f_dev, mu_dev, lam_dev, dj_dalpha_dev, dj_du_dev, dj_du_dev != nullptr, false));
+    CK(launch_adjoint_step_any(ctx, f_dev, ctx->nx, mu_dev, lam_dev, dj_dalpha_dev, dj_du_dev, dj_du_dev != nullptr, false));
     return DUGKS_OK;
 }
 
@@ -1863,9 +1908,14 @@ dugks_status dugks_adjoint(dugks_ctx* ctx, const void* phi0_dev, long long nstep
     if (st != DUGKS_OK) return st;
     const long long K = std::min<long long>(checkpoint_every, std::max<long long>(nsteps, 1));
     const long long nseg = nsteps == 0 ? 0 : (nsteps + K - 1) / K;
-    // states of 256-byte-aligned size in one workspace: nseg checkpoints, K segment states, two lambdas
-    const size_t sbytes = (size_t(Q) * ctx->nx * ctx->ny * ctx->elem + 255) / 256 * 256;
-    const size_t need = sbytes * size_t(nseg + K + 2);
+    // one workspace: the states at the segment starts after the first (the first is the context's own
+    // state buffer) and the states of a segment after its start, laid out like the context's
+    // buffers, and two lambdas
+    const size_t sbytes = size_t(Q) * ctx->plane * ctx->elem;
+    const size_t lbytes = (size_t(Q) * ctx->nx * ctx->ny * ctx->elem + 255) / 256 * 256;
+    const long long nck = std::max<long long>(nseg - 1, 0), nst = nck + K - 1;
+    const size_t at_lam = (sbytes * size_t(nst) + 255) / 256 * 256;
+    const size_t need = at_lam + 2 * lbytes;
     if (need > ctx->adj_ws_bytes) {
         if (ctx->adj_ws) {
             cudaStreamSynchronize(ctx->stream);
@@ -1881,22 +1931,51 @@ dugks_status dugks_adjoint(dugks_ctx* ctx, const void* phi0_dev, long long nstep
         ctx->adj_ws_bytes = need;
     }
     unsigned char* ws = static_cast<unsigned char*>(ctx->adj_ws);
-    std::vector<void*> ckpt(size_t(nseg), nullptr), seg(size_t(K), nullptr);
-    for (long long q = 0; q < nseg; ++q) ckpt[size_t(q)] = ws + size_t(q) * sbytes;
-    for (long long q = 0; q < K; ++q) seg[size_t(q)] = ws + size_t(nseg + q) * sbytes;
-    void* lam[2] = {ws + size_t(nseg + K) * sbytes, ws + size_t(nseg + K + 1) * sbytes};
+    std::vector<void*> state(size_t(nst) + 1, nullptr);  // [0]: step 0, [1 .. nck]: segment starts, then the segment
+    for (long long q = 0; q < nst; ++q) state[size_t(q) + 1] = ws + size_t(q) * sbytes;
+    void* const* seg = state.data() + nck;  // seg[q], q >= 1: the state q steps into the segment
+    void* lam[2] = {ws + at_lam, ws + at_lam + lbytes};
     auto fail = [&](cudaError_t e, const char* what) {
         dugks_status s = cuda_fail(ctx, e, what);
         cudaStreamSynchronize(ctx->stream);
         return s;
     };
     cudaError_t e;
-    // forward sweep, keeping one state per segment
     if ((st = dugks_init_phi(ctx, phi0_dev)) != DUGKS_OK) return st;
-    for (long long s = 0; s < nseg; ++s) {
-        if ((st = dugks_save_state(ctx, ckpt[s])) != DUGKS_OK) return st;
-        if ((st = dugks_step(ctx, std::min(K, nsteps - s * K))) != DUGKS_OK) return st;
-    }
+    state[0] = ctx->buf[ctx->cur];
+    std::vector<CUtensorMap> map(state.size());
+    if (ctx->kernel == DUGKS_KERNEL_FUSED && (st = make_state_maps(ctx, state.data(), int(state.size()), map.data())) != DUGKS_OK)
+        return st;
+    auto step = [&](long long from, long long to) {  // one row-marching step between two states
+        return launch_step_any(ctx, StepIO{state[size_t(from)], state[size_t(to)], &map[size_t(from)]});
+    };
+    // n steps from state `from` to state `to`, the states in between (keep) in seg[1 .. n - 1], or
+    // there only for a while; a resident launch keeps them as it goes
+    auto advance = [&](long long from, long long to, long long n, bool keep) -> cudaError_t {
+        const long long chunk = resident_chunk(ctx);
+        if (chunk > 0) {
+            cudaError_t r = cudaSuccess;
+            const void* in = state[size_t(from)];
+            for (long long s = 0, m; s < n && r == cudaSuccess; s += m) {
+                m = std::min(chunk, n - s);
+                void* out = s + m == n || !keep ? state[size_t(to)] : seg[s + m];
+                r = run_resident(ctx, int(m), in, out, keep ? seg[s + 1] : nullptr);
+                in = out;
+            }
+            if (r != cudaErrorCooperativeLaunchTooLarge) return r;
+        }
+        cudaError_t r = cudaSuccess;
+        long long at = from;
+        for (long long s = 1; s <= n && r == cudaSuccess; ++s) {
+            const long long next = s == n ? to : nck + (keep ? s : 1 + ((s - 1) & 1));
+            r = step(at, next);
+            at = next;
+        }
+        return r;
+    };
+    // forward sweep to the start of the last segment, keeping the state at the start of each
+    for (long long s = 0; s + 1 < nseg; ++s)
+        if ((e = advance(s, s + 1, K, false)) != cudaSuccess) return fail(e, "forward sweep");
     if ((e = cudaMemsetAsync(ctx->adj_dalpha, 0, 3 * sizeof(double), ctx->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(ctx->adj_partial, 0, 3 * sizeof(double) * size_t(adj_partials(ctx)), ctx->stream)) !=
             cudaSuccess)
@@ -1916,13 +1995,10 @@ dugks_status dugks_adjoint(dugks_ctx* ctx, const void* phi0_dev, long long nstep
     // reverse sweep: recompute each segment from its checkpoint, then step the adjoint back through it
     for (long long s = nseg - 1; s >= 0; --s) {
         const long long ns = std::min(K, nsteps - s * K);
-        if ((st = dugks_load_state(ctx, ckpt[s])) != DUGKS_OK) return st;
-        for (long long q = 0; q < ns; ++q) {
-            if ((st = dugks_save_state(ctx, seg[q])) != DUGKS_OK) return st;
-            if (q + 1 < ns && (st = dugks_step(ctx, 1)) != DUGKS_OK) return st;
-        }
+        if (ns > 1 && (e = advance(s, nck + ns - 1, ns - 1, true)) != cudaSuccess) return fail(e, "recomputed segment");
         for (long long q = ns - 1; q >= 0; --q) {
-            if ((e = launch_adjoint_step_any(ctx, seg[q], lam[cur], lam[1 - cur], nullptr, nullptr, want_u, true)) !=
+            const void* f = q == 0 ? state[size_t(s)] : seg[q];
+            if ((e = launch_adjoint_step_any(ctx, f, ctx->pitch, lam[cur], lam[1 - cur], nullptr, nullptr, want_u, true)) !=
                 cudaSuccess)
                 return fail(e, "adjoint step");
             cur ^= 1;

@@ -79,7 +79,10 @@ struct ResConsts {
 
 template <typename T>
 struct ResArgs {
-    T* f;                    // [9][ny][pitch]: read at the start, written at the end
+    const T* fin;            // state [9][ny][pitch] read at the start
+    T* fout;                 // state written at the end (may be fin: a CTA touches its own cells only)
+    T* rec;                  // if set, the states after steps 1 .. nsteps - 1, rstride elements apart
+    long long rstride;
     long long pitch, plane;
     int nx, ny, xper, yper;
     const FaceM<T>*fx, *fy;  // faces -1 .. n+1 at index f + 1
@@ -479,7 +482,7 @@ __global__ void __launch_bounds__(kResThreads<T>, 1)
     for (int i = tid; i < 3 * NE; i += NT) sM[i] = T(0);
     for (int i = tid; i < ncell; i += NT) {
         const int ly = i / tx, lx = i - ly * tx, u = ly * UX + lx;
-        const T* src = a.f + (long long)(y0 + ly) * a.pitch + x0 + lx;
+        const T* src = a.fin + (long long)(y0 + ly) * a.pitch + x0 + lx;
 #pragma unroll
         for (int q = 0; q < 4; ++q) sU[q * NU + u] = pk(src[PA(q) * a.plane], src[PB(q) * a.plane]);
         sZ[u] = src[0];
@@ -577,6 +580,15 @@ __global__ void __launch_bounds__(kResThreads<T>, 1)
             PT F[4], P[4], U[4];
             state_of(u, lx, F);
             const T Fz = sZ[u];
+            if (a.rec && step > 0) {
+                T* dst = a.rec + (step - 1) * a.rstride + (long long)(y0 + ly) * a.pitch + x0 + lx;
+                dst[0] = Fz;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    dst[PA(q) * a.plane] = F[q].v.x;
+                    dst[PB(q) * a.plane] = F[q].v.y;
+                }
+            }
             // P (Eq. 2.21), ftilde^+ (Eq. 2.23), as sv_cell
             const PT s4 = (F[0] + F[1]) + (F[2] + F[3]);
             const T phi = Fz + (s4.v.x + s4.v.y);
@@ -724,7 +736,7 @@ __global__ void __launch_bounds__(kResThreads<T>, 1)
         const int ly = i / tx, lx = i - ly * tx, u = ly * UX + lx;
         PT F[4];
         state_of(u, lx, F);
-        T* dst = a.f + (long long)(y0 + ly) * a.pitch + x0 + lx;
+        T* dst = a.fout + (long long)(y0 + ly) * a.pitch + x0 + lx;
         dst[0] = sZ[u];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
