@@ -314,6 +314,18 @@ struct InitOp {
         return cudaGetLastError();
     }
 };
+// phi alone where its cells can be taken four at a time
+struct PhiOnlyOp {
+    dugks_3d_ctx* ctx;
+    void* phi;
+    template <typename T, int QQ, int NC, int NW>
+    cudaError_t operator()() const {
+        const long long n = (long long)ctx->nx * ctx->ny * ctx->nz;
+        const unsigned blocks = unsigned(std::min<long long>((n / 4 + 255) / 256, 1 << 20));
+        phi3<T, QQ><<<blocks, 256, 0, ctx->stream>>>(static_cast<const T*>(ctx->buf[ctx->cur]), static_cast<T*>(phi), n);
+        return cudaGetLastError();
+    }
+};
 struct PhiOp {
     dugks_3d_ctx* ctx;
     void* phi;
@@ -545,6 +557,11 @@ dugks_status dugks_3d_step(dugks_3d_ctx* ctx, long long n) {
 dugks_status dugks_3d_get_phi(dugks_3d_ctx* ctx, void* phi_dev_out, double* mass_out) {
     if (!ctx) return DUGKS_ERR_ARG;
     Guard3 g(ctx->device);
+    const long long cells = (long long)ctx->nx * ctx->ny * ctx->nz;
+    if (!mass_out && phi_dev_out && cells % 4 == 0 && reinterpret_cast<uintptr_t>(phi_dev_out) % 16 == 0) {
+        CK3(dispatch3(ctx, PhiOnlyOp{ctx, phi_dev_out}));
+        return DUGKS_OK;
+    }
     CK3(dispatch3(ctx, PhiOp{ctx, phi_dev_out}));
     if (mass_out) {
         CK3(cudaMemcpyAsync(mass_out, ctx->mass_dev, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));

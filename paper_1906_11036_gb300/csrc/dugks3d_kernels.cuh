@@ -761,6 +761,25 @@ __global__ void __launch_bounds__(NW * 32, 1)
     }
 }
 
+// phi = sum_i ftilde_i of n cells, four at a time (V = float4 or a pair of double2: n a multiple of
+// four, phi aligned to 16 bytes)
+template <typename T, int QQ>
+__global__ void __launch_bounds__(256) phi3(const T* __restrict__ f, T* __restrict__ phi, long long n) {
+    struct __align__(16) V4 { T v[4]; };
+    for (long long c = 4 * (blockIdx.x * (long long)blockDim.x + threadIdx.x); c < n; c += 4LL * gridDim.x * blockDim.x) {
+        V4 s;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s.v[e] = T(0);
+#pragma unroll
+        for (int i = 0; i < QQ; ++i) {
+            const V4 x = *reinterpret_cast<const V4*>(f + i * n + c);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s.v[e] += x.v[e];
+        }
+        *reinterpret_cast<V4*>(phi + c) = s;
+    }
+}
+
 // phi = sum_i ftilde_i (optional output) and per-block partial sums of |V| phi in double
 template <typename T, int QQ>
 __global__ void __launch_bounds__(256) phi_mass3(const T* __restrict__ f, T* __restrict__ phi, int nx, int ny, int nz,

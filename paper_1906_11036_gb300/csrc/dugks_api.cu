@@ -864,15 +864,59 @@ cudaError_t run_resident(dugks_ctx* ctx, int n, const void* in, void* out, void*
     return e;
 }
 
+// grid of the field passes over rows of nx elements, and whether rows of nx elements from p on can be
+// accessed by 16 bytes
+dim3 field_grid(int nx, int rows) {
+    return dim3(unsigned(std::min((nx + 4 * kFieldX - 1) / (4 * kFieldX), 65535)),
+                unsigned(std::min((rows + kFieldY - 1) / kFieldY, 65535)));
+}
+bool rows_by_16(const void* p, size_t elem, int nx) {
+    return reinterpret_cast<uintptr_t>(p) % 16 == 0 && nx % 4 == 0 && elem >= 4;
+}
+
 template <typename T, typename Tin>
 cudaError_t launch_init(dugks_ctx* ctx, const Tin* phi0) {
-    const long long n = (long long)ctx->nx * ctx->ny;
-    const int blocks = int(std::min<long long>((n + 255) / 256, 65535));
     T* f = static_cast<T*>(ctx->buf[ctx->cur]);
-    // the initialisation is not on the hot path: always the generic polynomial degree
-    init_kernel<T, NC_LARGE, Tin><<<blocks, 256, 0, ctx->stream>>>(phi0, f, ctx->nx, ctx->ny, ctx->pitch, ctx->plane,
-                                                                  make_consts<T, NC_LARGE>(ctx),
-                                                                  ctx->feq_check ? ctx->err_dev : nullptr);
+    int* err = ctx->feq_check ? ctx->err_dev : nullptr;
+    const dim3 grid = field_grid(ctx->nx, ctx->ny), block(kFieldX, kFieldY);
+    const int vec = rows_by_16(phi0, sizeof(Tin), ctx->nx);
+    auto go = [&](auto nc) {
+        constexpr int NC = decltype(nc)::value;
+        init_kernel<T, NC, Tin><<<grid, block, 0, ctx->stream>>>(phi0, f, ctx->nx, ctx->ny, ctx->pitch, ctx->plane,
+                                                                make_consts<T, NC>(ctx), err, vec);
+    };
+    if (ctx->nc == 3) go(std::integral_constant<int, 3>{});
+    else if (ctx->nc == 4) go(std::integral_constant<int, 4>{});
+    else go(std::integral_constant<int, NC_LARGE>{});
+    return cudaGetLastError();
+}
+
+// phi alone, without the mass
+template <typename T>
+cudaError_t launch_phi_only(dugks_ctx* ctx, T* phi) {
+    phi_kernel<T><<<field_grid(ctx->nx, ctx->ny), dim3(kFieldX, kFieldY), 0, ctx->stream>>>(
+        static_cast<const T*>(ctx->buf[ctx->cur]), phi, ctx->nx, ctx->ny, ctx->pitch, ctx->plane,
+        rows_by_16(phi, sizeof(T), ctx->nx));
+    return cudaGetLastError();
+}
+
+// The state's Q ny rows between the context's pitch and contiguous rows of the caller's
+template <typename T>
+cudaError_t copy_state(dugks_ctx* ctx, const void* src, long long spitch, void* dst, long long dpitch) {
+    const size_t row = size_t(ctx->nx) * sizeof(T);
+    if (spitch == dpitch)
+        return cudaMemcpyAsync(dst, src, row * Q * ctx->ny, cudaMemcpyDeviceToDevice, ctx->stream);
+    const long long rows = (long long)Q * ctx->ny;
+    if (rows > INT_MAX / 2)
+        return cudaMemcpy2DAsync(dst, size_t(dpitch) * sizeof(T), src, size_t(spitch) * sizeof(T), row, size_t(rows),
+                                 cudaMemcpyDeviceToDevice, ctx->stream);
+    const dim3 grid = field_grid(ctx->nx, int(rows)), block(kFieldX, kFieldY);
+    const T* from = static_cast<const T*>(src);
+    T* to = static_cast<T*>(dst);
+    if (rows_by_16(src, sizeof(T), ctx->nx) && rows_by_16(dst, sizeof(T), ctx->nx))
+        copy_rows_kernel<T, true><<<grid, block, 0, ctx->stream>>>(from, to, ctx->nx, int(rows), spitch, dpitch);
+    else
+        copy_rows_kernel<T, false><<<grid, block, 0, ctx->stream>>>(from, to, ctx->nx, int(rows), spitch, dpitch);
     return cudaGetLastError();
 }
 
@@ -1659,14 +1703,18 @@ dugks_status dugks_step(dugks_ctx* ctx, long long n) {
 dugks_status dugks_get_phi(dugks_ctx* ctx, void* phi_dev_out, double* mass_out) {
     if (!ctx) return DUGKS_ERR_ARG;
     DeviceGuard guard(ctx->device);
+    if (!mass_out) {
+        if (phi_dev_out)
+            CK(ctx->precision == 32 ? launch_phi_only(ctx, static_cast<float*>(phi_dev_out))
+                                    : launch_phi_only(ctx, static_cast<double*>(phi_dev_out)));
+        return DUGKS_OK;
+    }
     cudaError_t e = ctx->precision == 32 ? launch_phi<float, float>(ctx, static_cast<float*>(phi_dev_out))
                                          : launch_phi<double, double>(ctx, static_cast<double*>(phi_dev_out));
     CK(e);
-    if (mass_out) {
-        CK(cudaMemcpyAsync(mass_out, ctx->mass_dev, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-        CK(cudaStreamSynchronize(ctx->stream));
-        if (!std::isfinite(*mass_out)) return DUGKS_ERR_NONFINITE;
-    }
+    CK(cudaMemcpyAsync(mass_out, ctx->mass_dev, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    if (!std::isfinite(*mass_out)) return DUGKS_ERR_NONFINITE;
     return DUGKS_OK;
 }
 
@@ -1690,16 +1738,16 @@ dugks_status dugks_get_phi_host(dugks_ctx* ctx, double* phi_host_out, double* ma
 dugks_status dugks_save_state(dugks_ctx* ctx, void* f_dev_out) {
     if (!ctx || !f_dev_out) return DUGKS_ERR_ARG;
     DeviceGuard guard(ctx->device);
-    CK(cudaMemcpy2DAsync(f_dev_out, size_t(ctx->nx) * ctx->elem, ctx->buf[ctx->cur], size_t(ctx->pitch) * ctx->elem,
-                         size_t(ctx->nx) * ctx->elem, size_t(Q) * ctx->ny, cudaMemcpyDeviceToDevice, ctx->stream));
+    CK(ctx->precision == 32 ? copy_state<float>(ctx, ctx->buf[ctx->cur], ctx->pitch, f_dev_out, ctx->nx)
+                            : copy_state<double>(ctx, ctx->buf[ctx->cur], ctx->pitch, f_dev_out, ctx->nx));
     return DUGKS_OK;
 }
 
 dugks_status dugks_load_state(dugks_ctx* ctx, const void* f_dev_in) {
     if (!ctx || !f_dev_in) return DUGKS_ERR_ARG;
     DeviceGuard guard(ctx->device);
-    CK(cudaMemcpy2DAsync(ctx->buf[ctx->cur], size_t(ctx->pitch) * ctx->elem, f_dev_in, size_t(ctx->nx) * ctx->elem,
-                         size_t(ctx->nx) * ctx->elem, size_t(Q) * ctx->ny, cudaMemcpyDeviceToDevice, ctx->stream));
+    CK(ctx->precision == 32 ? copy_state<float>(ctx, f_dev_in, ctx->nx, ctx->buf[ctx->cur], ctx->pitch)
+                            : copy_state<double>(ctx, f_dev_in, ctx->nx, ctx->buf[ctx->cur], ctx->pitch));
     ctx->steps_done = 0;
     ctx->src_first = true;  // the state carries no source history; time is kept
     ctx->tbase = ctx->t;
