@@ -86,6 +86,8 @@ struct dugks_ctx {
     int nseg_sp_src = 0;
     SegPlan sp{1, 0, 1};  // step_vp: long segments first, then short ones
     ResPlan res, res_src;  // the resident step without and with source terms
+    FlowPlan flow{0, 0, 0, nullptr};  // flow_vp (rows = 0: not taken)
+    bool flow_plain = false;          // with the interior variant
     long long steps_done = 0;
     // adjoint work buffers (allocated on first use)
     void* adj_ax = nullptr;
@@ -847,6 +849,63 @@ cudaError_t launch_resident_any(dugks_ctx* ctx, int n, const void* in, void* out
     return ctx->precision == 32 ? pick(float(0)) : pick(double(0));
 }
 
+// Tiles of flow_vp per resident warp, and rows per tile at least.  More tiles than warps hide the start
+// and the end of a tile behind others, but each passes two rows more than it owns (us per step for
+// 1.4, 1.7, 2.0, 2.8 tiles per warp: 2048^2 tanh mesh 59.9, 60.8, 61.7, 67.3; 2048^2 periodic 74.0,
+// 64.8, 64.2, 69.3; 1024^2 23.1, 21.2, 21.7, 21.8).  On grids too small for that, short tiles keep the
+// chain of a step short (800x700: 10 rows 21.7, 8 20.2, 6 17.7, 4 16.4).
+// One launch per step (step_vp) took 64.4, 76.1, 25.8 and 20.6 us on these grids.
+#ifndef DUGKS_FLOW_WAVES
+#define DUGKS_FLOW_WAVES 1.75
+#endif
+#ifndef DUGKS_FLOW_MIN_ROWS
+#define DUGKS_FLOW_MIN_ROWS 4
+#endif
+// rows per tile from which the interior variant of the row routine pays (see step_vp)
+#ifndef DUGKS_FLOW_PLAIN_ROWS
+#define DUGKS_FLOW_PLAIN_ROWS 24
+#endif
+constexpr int kFlowChunk = 256;  // steps per launch at most
+
+template <int NC>
+void* flow_fn(bool plain) {
+    return plain ? reinterpret_cast<void*>(&flow_vp<NC, true>) : reinterpret_cast<void*>(&flow_vp<NC, false>);
+}
+
+// Every FP32 grid that does not take the resident step takes flow_vp for calls of more than one step
+// (equilibria of degree <= 3, no source terms); tiles are counted in 32 bits.
+dugks_status plan_flow(dugks_ctx* ctx) {
+    if (ctx->precision != 32 || ctx->nc == NC_LARGE) return DUGKS_OK;
+    const double slots = double(ctx->sms) * ctx->occupancy;
+    const long long want = std::max<long long>(1, (long long)(DUGKS_FLOW_WAVES * slots / ctx->nstrips));
+    FlowPlan f{0, 0, ctx->nstrips, nullptr};
+    f.rows = int(std::max<long long>(std::min(DUGKS_FLOW_MIN_ROWS, ctx->ny), (ctx->ny + want - 1) / want));
+    f.nseg = (ctx->ny + f.rows - 1) / f.rows;
+    if ((long long)f.nstrips * f.nseg > INT_MAX / kFlowChunk) return DUGKS_OK;
+    ctx->flow_plain = f.rows >= DUGKS_FLOW_PLAIN_ROWS;
+    void* fn = ctx->nc == 3 ? flow_fn<3>(ctx->flow_plain) : flow_fn<4>(ctx->flow_plain);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(fused_smem(ctx)));
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
+    ctx->flow = f;
+    return DUGKS_OK;
+}
+size_t flow_bytes(const FlowPlan& f) { return f.rows ? (1 + size_t(f.nstrips) * f.nseg) * sizeof(unsigned) : 0; }
+
+template <int NC>
+cudaError_t launch_flow(dugks_ctx* ctx, int n) {
+    cudaError_t e = cudaMemsetAsync(ctx->flow.sync, 0, flow_bytes(ctx->flow), ctx->stream);
+    if (e != cudaSuccess) return e;
+    const unsigned grid = unsigned(n) * unsigned(ctx->flow.nstrips) * unsigned(ctx->flow.nseg);
+    const int c = ctx->cur;
+    if (ctx->flow_plain)
+        flow_vp<NC, true><<<grid, 32, fused_smem(ctx), ctx->stream>>>(ctx->tmap[c], ctx->tmap[c ^ 1], make_args<float, NC>(ctx, c),
+                                                                     make_constsp<NC>(ctx), ctx->rowy, ctx->flow, ctx->stages);
+    else
+        flow_vp<NC, false><<<grid, 32, fused_smem(ctx), ctx->stream>>>(ctx->tmap[c], ctx->tmap[c ^ 1], make_args<float, NC>(ctx, c),
+                                                                      make_constsp<NC>(ctx), ctx->rowy, ctx->flow, ctx->stages);
+    return cudaGetLastError();
+}
+
 // steps a resident launch may take (0: the grid runs the row-marching kernels)
 long long resident_chunk(const dugks_ctx* ctx) {
     if ((ctx->nsrc > 0 ? ctx->res_src : ctx->res).ntx == 0) return 0;
@@ -1528,8 +1587,11 @@ static dugks_status create_ctx(const dugks_mesh* mesh, const dugks_vset* vset, c
         free_ctx(ctx);
         return r;
     };
-    if (stepped_alone && ctx->kernel == DUGKS_KERNEL_FUSED && (st = plan_resident(ctx, 0, ctx->res)) != DUGKS_OK)
-        return fail(st);
+    if (ctx->kernel == DUGKS_KERNEL_FUSED) {
+        if ((st = plan_fused(ctx)) != DUGKS_OK) return fail(st);
+        if (stepped_alone && (st = plan_resident(ctx, 0, ctx->res)) != DUGKS_OK) return fail(st);
+        if (stepped_alone && ctx->res.ntx == 0 && (st = plan_flow(ctx)) != DUGKS_OK) return fail(st);
+    }
 
     const int lane = 128 / int(ctx->elem);  // rows padded to 128 bytes
     ctx->pitch = ((long long)ctx->nx + lane - 1) / lane * lane;
@@ -1537,12 +1599,13 @@ static dugks_status create_ctx(const dugks_mesh* mesh, const dugks_vset* vset, c
     const size_t bytes = size_t(Q) * size_t(ctx->plane) * ctx->elem;  // (a multiple of 128)
 
     cudaError_t e;
-    for (int b = 0; b < 2; ++b) {  // the resident step's buffers lie behind the first state buffer
-        size_t n = bytes + (b == 0 ? resident_bytes(ctx, ctx->res) : 0);
+    for (int b = 0; b < 2; ++b) {  // the resident step's buffers or flow_vp's counts lie behind the first state buffer
+        size_t n = bytes + (b == 0 ? resident_bytes(ctx, ctx->res) + flow_bytes(ctx->flow) : 0);
         e = cudaMalloc(&ctx->buf[b], n);
-        if (e == cudaErrorMemoryAllocation && n > bytes) {  // no room for them: row-marching steps
+        if (e == cudaErrorMemoryAllocation && n > bytes) {  // no room for them: a launch per step
             cudaGetLastError();
             ctx->res = ResPlan();
+            ctx->flow.rows = 0;
             e = cudaMalloc(&ctx->buf[b], n = bytes);
         }
         if (e != cudaSuccess) { cuda_fail(ctx, e, "cudaMalloc(state)"); return fail(DUGKS_ERR_NOMEM); }
@@ -1550,6 +1613,7 @@ static dugks_status create_ctx(const dugks_mesh* mesh, const dugks_vset* vset, c
         if (e != cudaSuccess) return fail(cuda_fail(ctx, e, "cudaMemsetAsync"));
     }
     if (ctx->res.ntx) set_resident_buffers(ctx, ctx->res, static_cast<char*>(ctx->buf[0]) + bytes);
+    if (ctx->flow.rows) ctx->flow.sync = reinterpret_cast<unsigned*>(static_cast<char*>(ctx->buf[0]) + bytes);
     // metrics
     std::vector<double> dxw, dyw;
     auto upload = [&](void** dst, const void* src, size_t n) -> cudaError_t {
@@ -1602,8 +1666,6 @@ static dugks_status create_ctx(const dugks_mesh* mesh, const dugks_vset* vset, c
     if ((e = cudaMemsetAsync(ctx->err_dev, 0, sizeof(int), ctx->stream)) != cudaSuccess)
         return fail(cuda_fail(ctx, e, "cudaMemsetAsync(err)"));
     if (ctx->kernel == DUGKS_KERNEL_FUSED) {
-        st = plan_fused(ctx);
-        if (st != DUGKS_OK) return fail(st);
         st = make_state_maps(ctx, ctx->buf, 2, ctx->tmap);
         if (st != DUGKS_OK) return fail(st);
     }
@@ -1687,6 +1749,10 @@ dugks_status dugks_step(dugks_ctx* ctx, long long n) {
                 continue;
             }
             CK(e);
+        } else if (ctx->flow.rows > 0 && ctx->nsrc == 0 && n - s > 1) {
+            m = std::min<long long>(n - s, kFlowChunk);
+            CK(ctx->nc == 3 ? launch_flow<3>(ctx, int(m)) : launch_flow<4>(ctx, int(m)));
+            ctx->cur ^= int(m & 1);
         } else {
             m = 1;
             CK(launch_step_any(ctx, own_io(ctx)));

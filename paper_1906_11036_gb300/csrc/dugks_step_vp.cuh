@@ -415,6 +415,110 @@ __global__ void __launch_bounds__(32, DUGKS_SV_MIN_WARPS)
 
 
 // ---------------------------------------------------------------------------
+// many steps in one launch
+// ---------------------------------------------------------------------------
+//
+// With a launch per step the launch, the first loads and the last warps leave the GPU partly idle, on a
+// mid-sized grid, where a step is one wave of short segments, for a quarter of the step (1024^2:
+// 25.8 us, while a grid eight times as tall takes 18.9 us per 1024 rows).  flow_vp runs the tiles of many steps as one
+// sequence: a one-warp CTA takes the next tile from a counter, waits until the tile and its eight
+// neighbours have done the step before (their step counts, in device memory), runs the row routine
+// and raises its own count.  Tiles of a step start while others of the step before still run, so
+// there is no idle time between steps.  CTAs take tiles in sequence order, so a tile only ever waits
+// for tiles that running CTAs hold: the launch needs no co-residency.  A tile's stores are made
+// visible (fence) before its count rises, and the tile that reads the count orders its TMA loads,
+// which run in the asynchronous proxy, after it.  A tile overwrites the state of two steps before
+// only after its neighbours have counted the step that read it.  Waits are bounded; one that expires
+// sets the error word, which ends the CTAs that follow at once.  us per step, a launch per step ->
+// flow_vp: 1024^2 periodic 25.8 -> 21.2, 2048^2 periodic 76.1 -> 64, 2048^2 tanh mesh 64.4 -> 60.9,
+// 1500x900 with walls 32.0 -> 24.0, 800x700 20.6 -> 16.4.  (CTAs that stay and take their next tile
+// ahead of time were slower, 31 us at 1024^2: a tile taken ahead holds up its neighbours.)
+struct FlowPlan {
+    int rows, nseg, nstrips;
+    unsigned* sync;  // [0]: tiles taken; [1 + tile]: steps done (all zero at launch)
+};
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+template <int NC, bool IP>
+__global__ void __launch_bounds__(32, DUGKS_SV_MIN_WARPS)
+    flow_vp(const __grid_constant__ CUtensorMap t0, const __grid_constant__ CUtensorMap t1, const StepArgs<float, NC> a0,
+            const ConstsP<NC> k, const RowY* __restrict__ rw, const FlowPlan fp, const int S) {
+    using L = WarpLayout<float>;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + size_t(S) * L::STAGE_BYTES);
+    const int lane = threadIdx.x;
+    unsigned t = 0;
+    if (lane == 0) {
+        t = atomicAdd(fp.sync, 1u);
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&t0)) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&t1)) : "memory");
+        for (int q = 0; q < S; ++q) mbar_init(&bars[q], 1);
+        fence_mbar_init();
+    }
+    t = __shfl_sync(0xffffffffu, t, 0);
+    const unsigned tiles = unsigned(fp.nstrips) * unsigned(fp.nseg);
+    const unsigned step = t / tiles, tile = t - step * tiles;
+    const int sg = int(tile / unsigned(fp.nstrips)), st = int(tile) - sg * fp.nstrips;
+    const int xw = st * L::WI, y0 = sg * fp.rows, y1 = min(y0 + fp.rows, a0.ny);
+    bool ok = true;
+    if (step > 0 && lane < 9) {
+        int ns = st + lane % 3 - 1, ng = sg + lane / 3 - 1;
+        bool need = true;
+        if (ns < 0 || ns >= fp.nstrips) {
+            need = a0.xper;
+            ns = ns < 0 ? fp.nstrips - 1 : 0;
+        }
+        if (ng < 0 || ng >= fp.nseg) {
+            need = need && a0.yper;
+            ng = ng < 0 ? fp.nseg - 1 : 0;
+        }
+        if (need) {
+            const unsigned* p = fp.sync + 1 + ng * fp.nstrips + ns;
+            unsigned long long w0 = 0, w1;
+            for (unsigned spin = 1; ld_acquire(p) < step; ++spin) {
+                if ((spin & 63u) == 0) {
+                    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(w1));
+                    if (w0 == 0) w0 = w1;
+                    if (w1 - w0 > 2000000000ull || (*reinterpret_cast<volatile int*>(a0.err) & 1)) {
+                        ok = false;
+                        break;
+                    }
+                }
+            }
+        }
+    }
+    if (__any_sync(0xffffffffu, !ok)) {
+        if (lane == 0) atomicOr(a0.err, 1);
+        return;  // (no copy is in flight yet)
+    }
+    asm volatile("fence.proxy.async;" ::: "memory");
+    __syncwarp();
+    StepArgs<float, NC> a = a0;
+    if (step & 1u) {
+        a.fin = a0.fout;
+        a.fout = const_cast<float*>(a0.fin);
+    }
+    const CUtensorMap* tin = (step & 1u) ? &t1 : &t0;
+    const bool edge = xw - 1 < 0 || xw + L::WI >= a.nx;
+    const bool yg = !a.yper && (y0 == 0 || y1 == a.ny);
+    int ring = 0;
+    if (IP && !edge && !yg)
+        sv_rows<NC, true>(tin, a, k, rw, smem, bars, S, lane, xw, y0, y1, false, false, ring);
+    else
+        sv_rows<NC>(tin, a, k, rw, smem, bars, S, lane, xw, y0, y1, edge, yg, ring);
+    __syncwarp();  // every lane's stores come before the count
+    if (lane == 0) st_release(fp.sync + 1 + tile, step + 1u);
+}
+
+// ---------------------------------------------------------------------------
 // the same row routine with the source terms F and R
 // ---------------------------------------------------------------------------
 //

@@ -1,7 +1,8 @@
-"""The resident step (many steps per launch, tiles exchanging their rims) at
-the edges of its tiling: against the row-marching step, which the batched
-solver runs, bit for bit in FP32, and against the one-thread-per-cell kernel
-in FP64; replayed from a CUDA graph; grids just above its range."""
+"""The kernels that take many steps per launch, at the edges of their tiling:
+the resident step (tiles exchanging their rims) and the tile sequence of the
+row-marching step (tiles waiting for their neighbours), against the batched
+solver, which takes a launch per step, bit for bit in FP32; the resident step
+in FP64 against the one-thread-per-cell kernel; both replayed from a graph."""
 import numpy as np
 import pytest
 
@@ -23,8 +24,10 @@ def _gpu():
 
 
 # one row or column per tile, one tile more than there are SMs on an axis, tiles of uneven size, the
-# largest tiles of the range (x-fluxes in place), a grid just beyond it, lines of one cell
-SIZES = [(152, 1), (1, 153), (3, 305), (31, 33), (62, 31), (97, 620), (257, 509), (512, 512), (612, 617), (700, 610)]
+# largest tiles of the range (x-fluxes in place); then tile sequences: two strips, a clipped last tile,
+# tiles of the least height
+SIZES = [(152, 1), (1, 153), (3, 305), (31, 33), (62, 31), (97, 620), (257, 509), (512, 512), (612, 617), (700, 610),
+         (31, 20000), (5000, 90), (1021, 643), (1500, 601)]
 
 
 def _problem(nx, ny, xwall, ywall, linear=False):
@@ -76,12 +79,12 @@ def test_fp64_matches_the_cell_kernel(nx, ny):
         assert float((got - ref).norm() / ref.norm()) <= 1e-13
 
 
-@pytest.mark.parametrize("prec", [32, 64])
-def test_replay_from_a_graph(prec):
+@pytest.mark.parametrize("nx,ny,prec", [(70, 45, 32), (70, 45, 64), (900, 700, 32)])
+def test_replay_from_a_graph(nx, ny, prec):
     """A captured step call advances the state at every replay as direct calls do."""
     from paper_1906_11036_gb300.dugks import Solver
 
-    p, phi0 = _problem(70, 45, True, False)
+    p, phi0 = _problem(nx, ny, True, False)
     ref = _steps(p, phi0, prec, (3, 4, 4, 4))
     s = Solver(p, precision=prec)
     stream = torch.cuda.Stream()
