@@ -311,6 +311,9 @@ dugks_status dugks_batch_get_phi(dugks_batch *b, int i, void *phi_dev_out, doubl
 dugks_status dugks_batch_save_state(dugks_batch *b, int i, void *f_dev_out);
 /* Synchronise; DUGKS_ERR_TIMEOUT if a bounded device wait expired. */
 dugks_status dugks_batch_sync(dugks_batch *b);
+/* The CUDA stream the batch runs on (its own where the options gave none; library-owned
+ * then), so that a caller can order its own work with it; null for a null batch. */
+void *dugks_batch_stream(const dugks_batch *b);
 /* Autotuner: times steps_per_trial steps for each candidate tile height (rows
  * per tile, 8 ... 128), each without and with the split of every instance's
  * last rows (all but 0.8, 0.7 or 0.6 of them) into 8-row tiles queued after

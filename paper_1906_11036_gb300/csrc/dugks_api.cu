@@ -2251,6 +2251,8 @@ dugks_status dugks_batch_save_state(dugks_batch* b, int i, void* f_dev_out) {
     return dugks_save_state(b->ctx[size_t(i)], f_dev_out);
 }
 
+void* dugks_batch_stream(const dugks_batch* b) { return b ? b->stream : nullptr; }
+
 dugks_status dugks_batch_sync(dugks_batch* b) {
     if (!b) return DUGKS_ERR_ARG;
     DeviceGuard guard(b->device);

@@ -120,6 +120,8 @@ def library():
         L.dugks_batch_get_phi.argtypes = [vp, ctypes.c_int, vp, P(ctypes.c_double)]
         L.dugks_batch_save_state.argtypes = [vp, ctypes.c_int, vp]
         L.dugks_batch_sync.argtypes = [vp]
+        L.dugks_batch_stream.argtypes = [vp]
+        L.dugks_batch_stream.restype = vp
         L.dugks_batch_autotune.argtypes = [vp, ctypes.c_int, P(ctypes.c_int), P(ctypes.c_float)]
         L.dugks_batch_last_error.argtypes = [vp]
         L.dugks_batch_last_error.restype = ctypes.c_char_p
@@ -433,6 +435,10 @@ class BatchSolver:
         if st != OK:
             raise DugksError(st, "dugks_batch_create")
         self.h, self.L, self.n = h, L, n
+        # the stream the batch runs on, and two events that order it with the caller's stream around
+        # an initialisation
+        self._own = torch.cuda.ExternalStream(L.dugks_batch_stream(h), self.device)
+        self._ready, self._taken = torch.cuda.Event(), torch.cuda.Event()
 
     def _check(self, st, where):
         if st != OK:
@@ -453,8 +459,13 @@ class BatchSolver:
         p = self.problems[i]
         t = self.torch.as_tensor(phi0).to(device=self.device, dtype=self.torch.float32).contiguous()
         assert tuple(t.shape) == (p.ny, p.nx)
+        # the batch's stream waits for phi0, the caller's for its use (phi0 may be changed or freed then)
+        caller = self.torch.cuda.current_stream(self.device)
+        self._ready.record(caller)
+        self._own.wait_event(self._ready)
         self._check(self.L.dugks_batch_init_phi(self.h, int(i), ctypes.c_void_p(t.data_ptr())), "dugks_batch_init_phi")
-        self.sync()
+        self._taken.record(self._own)
+        caller.wait_event(self._taken)
 
     def step(self, n: int = 1):
         self._check(self.L.dugks_batch_step(self.h, int(n)), "dugks_batch_step")
