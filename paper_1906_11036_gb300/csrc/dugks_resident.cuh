@@ -325,6 +325,78 @@ __device__ __forceinline__ void res_march(const ResConsts<T, NC>& k, const Pair<
     }
 }
 
+// Step 1 of one tile of at most 32 cells in FP64: warps 0 .. 3 take eight cells each (c: this lane's
+// cell, bit 31 set where it has one), lane group q = lane / 8 the pair q; sums over the pairs go
+// through shuffles.  The FP64 pipe of a quarter of an SM takes 64 clocks for an instruction of a warp
+// whatever its active lanes, so one warp alone needs about 75 x 64 clocks for its cells while the
+// other three quarters idle; split, each quarter runs about 28 (64^2: 5.9 -> 4.8 us per step).
+// hq: the lane's pair of hbp; no source terms, no wall cells.
+template <typename T, int NC, typename Slot>
+__device__ __forceinline__ void res_cell_parts(const ResArgs<T>& a, const ResConsts<T, NC>& k, const Vec2<T>* hq, Pair<T>* sP,
+                                               T* sM, Pair<T>* sU, T* sZ, const Pair<T>* sD, const T* sCx, unsigned c,
+                                               int NE, int NU, int EX, int UX, int lane, int warp, int step, int x0, int y0,
+                                               Slot&& slot, unsigned tag) {
+    if constexpr (sizeof(T) == 8 && NC <= 4) {
+        using PT = Pair<T>;
+        if (warp >= 4) return;
+        const int q = lane >> 3, lx = int(c & 0xfffu), ly = int(c >> 12 & 0xfffu);
+        const int u = ly * UX + lx, e = (ly + 1) * EX + lx + 1;
+        const bool live = c >> 31;
+        auto over_pairs = [&](T x) {
+            x += __shfl_xor_sync(0xffffffffu, x, 8);
+            return x + __shfl_xor_sync(0xffffffffu, x, 16);
+        };
+        PT F = sU[q * NU + u];
+        if (!a.seq) {  // the x-fluxes of the step before (pair 1 has none)
+            const T r = sCx[2 * (lx + 1) + 1], rx = q == 1 ? T(0) : (q == 3 ? -r : r);
+            F = fma2(pk(-rx, rx), sD[max(q - 1, 0) * NU + u], F);
+        }
+        const T Fz = sZ[u];
+        if (a.rec && step > 0 && live) {
+            T* dst = a.rec + (step - 1) * a.rstride + (long long)(y0 + ly) * a.pitch + x0 + lx;
+            if (q == 0) dst[0] = Fz;
+            const int pa = q == 0 ? PA(0) : q == 1 ? PA(1) : q == 2 ? PA(2) : PA(3);
+            const int pb = q == 0 ? PB(0) : q == 1 ? PB(1) : q == 2 ? PB(2) : PB(3);
+            dst[pa * a.plane] = F.v.x;
+            dst[pb * a.plane] = F.v.y;
+        }
+        const T phi = Fz + over_pairs(F.v.x + F.v.y);
+        PT h{hq[NC - 1]};
+#pragma unroll
+        for (int m = NC - 2; m >= 0; --m) h = fma2(h, pk(phi, phi), PT{hq[m]});
+        const PT P = fma2(pk(k.a_bp, k.a_bp), F, h);
+        if (live) sP[q * NE + e] = P;
+        if (live && q == 0) sM[e] = phi;
+        __syncwarp();
+        // the words of the eight cells, six each, as 32-bit halves of the values just stored
+        for (int i = lane; i < 48; i += 32) {
+            const unsigned oc = __shfl_sync(i < 32 ? 0xffffffffu : 0x0000ffffu, c, i / 6);
+            if (!(oc >> 31) || !(oc >> 24 & 1u)) continue;
+            const int olx = int(oc & 0xfffu), oly = int(oc >> 12 & 0xfffu), oe = (oly + 1) * EX + olx + 1, w = i % 6;
+            unsigned v[3];
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                const int half = 3 * w + m, d = half >> 1;  // value d: pair d / 2, component d % 2; 8: phi
+                const unsigned* src = d < 8 ? reinterpret_cast<const unsigned*>(sP + (d >> 1) * NE + oe) + 2 * (d & 1)
+                                            : reinterpret_cast<const unsigned*>(sM + oe);
+                v[m] = src[half & 1];
+            }
+            st_word(slot(olx, oly) + w, v[0], v[1], v[2], tag);
+        }
+        const T Pz = fma(k.a_bp, Fz, fma(k.b_bp, phi, -over_pairs(h.v.x + h.v.y)));
+        const T d = P.v.x - P.v.y;
+        const T mx = over_pairs(q == 1 ? T(0) : (q == 3 ? -d : d)), my = over_pairs(q == 0 ? T(0) : d);
+        if (live) {
+            sU[q * NU + u] = fma2(pk(k.third, k.third), P - F, P);
+            if (q == 0) {
+                sM[NE + e] = mx;
+                sM[2 * NE + e] = my;
+                sZ[u] = fma(k.third, Pz - Fz, Pz);
+            }
+        }
+    }
+}
+
 #ifndef DUGKS_RES_THREADS32
 #define DUGKS_RES_THREADS32 512
 #endif
@@ -568,12 +640,25 @@ __global__ void __launch_bounds__(kResThreads<T>, 1)
     // most tiles give a warp one group and a thread one cell: these are worked out once
     const March m_first = march_of(min(warp, gyn + gxn - 1)), mx_first = march_of(gyn + min(warp, gxn - 1));
     const unsigned c_first = tid < ncell ? sI[tid] : 0u;
+    // FP64 tiles of one warp's cells: four warps take eight cells each, a lane per pair
+    constexpr bool kSplit = sizeof(T) == 8 && NC <= 4 && !SRC;
+    const bool split = kSplit && ncell <= 32 && nwarps >= 4 && !__syncthreads_or(tid < ncell && (c_first >> 25));
+    const int i_split = warp * 8 + (lane & 7);
+    const unsigned c_split = split && warp < 4 && i_split < ncell ? sI[i_split] | 1u << 31 : 0u;
+    Vec2<T> hq[kSplit ? NC : 1];
+    if constexpr (kSplit)
+#pragma unroll
+        for (int m = 0; m < NC; ++m) hq[m] = k.hbp[lane >> 3][m];
     bool fail = false;
     for (int step = 0; step < a.nsteps; ++step) {
         const unsigned tag = tag0 + unsigned(step) + 1u;
         uint4* pub = own + (tag & 1u) * xbuf;
+        if (split) {
+            res_cell_parts<T, NC>(a, k, hq, sP, sM, sU, sZ, sD, sCx, c_split, NE, NU, EX, UX, lane, warp, step, x0, y0,
+                                  [&](int lx, int ly) { return pub + slot_of(lx, ly, tx, ty) * W; }, tag);
+        }
         unsigned c = c_first;
-        for (int i = tid; i < ncell; i += NT) {
+        for (int i = split ? ncell : tid; i < ncell; i += NT) {
             if (i != tid) c = sI[i];
             const int lx = int(c & 0xfffu), ly = int(c >> 12 & 0xfffu);
             const int u = ly * UX + lx, e = (ly + 1) * EX + lx + 1;
@@ -601,10 +686,16 @@ __global__ void __launch_bounds__(kResThreads<T>, 1)
                 hs = hs + hq;
             }
             T Pz = fma(k.a_bp, Fz, fma(k.b_bp, phi, -(hs.v.x + hs.v.y)));
+            T m0 = phi, Uz;
+            auto relaxed = [&]() {  // ftilde^+ (Eq. 2.23)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) U[q] = fma2(th, P[q] - F[q], P[q]);
-            T Uz = fma(k.third, Pz - Fz, Pz);
-            T m0 = phi;
+                for (int q = 0; q < 4; ++q) U[q] = fma2(th, P[q] - F[q], P[q]);
+                Uz = fma(k.third, Pz - Fz, Pz);
+            };
+            // the neighbours' P leaves before ftilde^+ is formed: their waits end earlier (not with source
+            // terms, which enter both, nor at high degree, where the longer lives of P and F spill)
+            constexpr bool kEarly = !SRC && NC <= 4;
+            if constexpr (!kEarly) relaxed();
             if constexpr (SRC) {  // the source terms (as add_source_vp), phi^{n-1} kept in shared memory
                 const bool first = sa.first && step == 0;
                 const PT X = pk(phi, first ? phi : sH[u]);
@@ -633,9 +724,10 @@ __global__ void __launch_bounds__(kResThreads<T>, 1)
                 const PT p4 = (P[0] + P[1]) + (P[2] + P[3]);
                 m0 = Pz + (p4.v.x + p4.v.y);
             }
+            if (c & 1u << 24) res_publish(pub + slot_of(lx, ly, tx, ty) * W, P, m0, tag);
+            if constexpr (kEarly) relaxed();
             T mx, my;
             res_moments(P, mx, my);
-            if (c & 1u << 24) res_publish(pub + slot_of(lx, ly, tx, ty) * W, P, m0, tag);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 sP[q * NE + e] = P[q];
