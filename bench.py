@@ -4,8 +4,9 @@
                     [--workload nonuniform|burgers] [--substeps S]
 
 A bench step is one output interval of S DUGKS time steps (default 50) on
-the workload's full grid; every DUGKS time step is one launch of the fused
-step kernel, i.e. one pass of the whole method over the grid.
+the workload's full grid, advanced by one launch of the tile-sequence
+kernel (flow_vp) per 256 time steps; every DUGKS time step is one pass of the
+whole method over the grid.
 
 * value      : cell-velocity updates per second with the state resident in
                HBM (K intervals timed with CUDA events on the solver's stream).
@@ -16,7 +17,7 @@ step kernel, i.e. one pass of the whole method over the grid.
 * roofline   : the fused step kernel against the measured HBM copy
                bandwidth (and the nominal 7.9 TB/s); algorithmic bytes = read
                ftilde once + write once = 2 * 9 * sizeof(T) per cell; the
-               launch time is the looped interval time over its launches.
+               time of a step is the looped interval time over its time steps.
 * cpu_baseline (rank 0, N = 1): the FP64 CPU oracle on a bounded sample, on
                all host cores and on one, with the CPU model.
 * batched    : the 256-instance workload, 1000 steps as 20 graph replays,
@@ -49,10 +50,11 @@ METRIC = "DUGKS cell-velocity updates/sec and % HBM roofline (FP32, 1 GB300); ad
 UNIT = "cell-velocity updates/s"
 Q = 9
 PROFILE = os.path.join(ROOT, "profiles", "fused_step_nonuniform_2048.txt")
-# the files that define the FP32 step kernel (step_vp) and what it includes
+# the files that define the FP32 step kernels (flow_vp, step_vp) and what they include
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_1906_11036_gb300", "csrc", f)
                   for f in ("dugks_step_vp.cuh", "dugks_kernels.cuh", "dugks_device.cuh")]
 NOMINAL_HBM_GBS = 7900.0  # GB300 HBM3e, nominal
+FLOW_CHUNK = 256  # time steps per launch of flow_vp at most (kFlowChunk)
 
 
 def workload(name: str):
@@ -73,7 +75,7 @@ def kernel_source_hash() -> str:
 
 
 def profile_traffic(workload_name: str):
-    """dram bytes per launch from the committed ncu summary, if it was taken on
+    """dram bytes per time step from the committed ncu summary, if it was taken on
     the current kernel source and this workload; else None."""
     if not os.path.exists(PROFILE):
         return None
@@ -85,7 +87,7 @@ def profile_traffic(workload_name: str):
     if kv.get("kernel_source_hash") != kernel_source_hash() or kv.get("workload") != workload_name:
         return None
     try:
-        return float(kv["dram_bytes_per_launch_full_grid"])
+        return float(kv["dram_bytes_per_step_full_grid"])
     except (KeyError, ValueError):
         return None
 
@@ -729,7 +731,7 @@ def main():
     barrier()
     t_dev = ev0.elapsed_time(ev1) / 1e3
     solver.sync()
-    # ---- per-launch kernel duration (events around each launch) ------------------
+    # ---- single steps (events around each) ---------------------------------------
     nl = min(200, max(20, args.steps * S // 4))
     evs = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(nl)]
     for a, b in evs:
@@ -768,25 +770,25 @@ def main():
     e2e = replica_value(cvu_per_step * e2e_steps, world, t_e2e)
     peak, peak_kind = measured_peak()
     alg_bytes = 2 * Q * 4 * cells
-    # one launch per DUGKS time step: its duration from the looped timing (CUDA events around
-    # the K timed intervals of S launches each); the median of per-launch event pairs, which
-    # carry their own overhead, is reported beside it
-    launch_loop_s = t_dev / (args.steps * S)
-    achieved = alg_bytes / launch_loop_s / 1e9
+    # a DUGKS time step's duration from the looped timing (CUDA events around the K timed
+    # intervals of S time steps each); the median of event pairs around single steps (step_vp, a
+    # launch of its own), which carry their own overhead, is reported beside it
+    step_s = t_dev / (args.steps * S)
+    achieved = alg_bytes / step_s / 1e9
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": 1e3 * t_dev / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": config_dict(args, p),
         "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": 8 * cells, "d2h_bytes_per_step": 8 * cells + 8},
-        "gpu_launches": args.steps * S,
+        "gpu_launches": args.steps * -(-S // FLOW_CHUNK),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "traffic": profile_traffic(args.workload), "peak_kind": peak_kind,
                      "frac_of_nominal": achieved / NOMINAL_HBM_GBS, "nominal_peak": NOMINAL_HBM_GBS,
-                     "kernel": "step_vp", "kernel_ms": launch_loop_s * 1e3,
-                     "kernel_ms_from": "looped timing: interval time / launches",
+                     "kernel": "flow_vp", "kernel_ms": step_s * 1e3,
+                     "kernel_ms_from": "looped timing: interval time / time steps",
                      "kernel_ms_events": launch_s * 1e3,
-                     "algorithmic_bytes_per_launch": alg_bytes},
+                     "algorithmic_bytes_per_step": alg_bytes},
         "clocks": clk.summary(),
         "launch": {"block": info["block_threads"], "grid": info["grid_blocks"]},
     }

@@ -170,8 +170,10 @@ dugks_status dugks_init_phi(dugks_ctx *ctx, const void *phi0_dev);
 dugks_status dugks_init_phi_host(dugks_ctx *ctx, const double *phi0_host);
 
 /* Advance n >= 0 time steps (Eq. 2.12 with the interface flux of Eqs.
- * 2.19-2.22 and Eq. 2.9), asynchronously on the context's stream.  One kernel
- * launch per step; the two ftilde buffers alternate. */
+ * 2.19-2.22 and Eq. 2.9), asynchronously on the context's stream.  Grids whose
+ * state fits in the SMs' shared memory (about 630^2 cells in FP32, 435^2 in
+ * FP64) take up to 1024 steps per (cooperative) launch, or 32 with source
+ * terms; larger FP32 grids up to 256; otherwise one launch per step. */
 dugks_status dugks_step(dugks_ctx *ctx, long long n);
 
 /* phi = sum_i ftilde_i (text after Eq. 2.13) into phi_dev_out (device,
@@ -263,8 +265,8 @@ dugks_status dugks_set_feq_check(dugks_ctx *ctx, int on);
 
 /* Which kernel runs an FP32 adjoint step (a cross-check hook; results agree to
  * FP32 rounding).  DUGKS_ADJ_AUTO (the default): the row-marching kernel
- * (periodic or Dirichlet walls) on grids with nx a multiple of 4 from 1 M
- * cells (1024^2), else the tiled kernel; DUGKS_ADJ_TILED: always the tiled kernel;
+ * (periodic or Dirichlet walls) on grids with nx a multiple of 4 whose
+ * segments give every SM six warps (from about 320^2), else the tiled kernel; DUGKS_ADJ_TILED: always the tiled kernel;
  * DUGKS_ADJ_ROWS: the row-marching kernel wherever it applies, whatever the
  * size.  DUGKS_ERR_ARG for a null ctx or an unknown value. */
 enum { DUGKS_ADJ_AUTO = 0, DUGKS_ADJ_TILED = 1, DUGKS_ADJ_ROWS = 2 };

@@ -386,7 +386,7 @@ class Solver:
     def gradient(self, phi0, nsteps: int, grad_phiN, checkpoint_every: int = 20, with_u: bool = False):
         """(dJ/dphi0, dJ/dalpha) through nsteps steps, given dJ/dphi^N (checkpointed
         reverse sweep in the library); with_u: (dJ/dphi0, dJ/dalpha, (dJ/du_x,
-        dJ/du_y)).  Leaves the solver's state at an intermediate step."""
+        dJ/du_y)).  Leaves the solver's state at step 0 (initialised from phi0)."""
         t = self.torch
         phi0 = phi0.to(device=self.device, dtype=self.dtype).contiguous()
         g = grad_phiN.to(device=self.device, dtype=self.dtype).contiguous()
