@@ -556,7 +556,7 @@ void set_resident_buffers(const dugks_ctx* ctx, ResPlan& r, void* p) {
 // neighbours, keeps the row-marching kernels.  Up to that line the resident step was the faster one
 // wherever both were measured (us per step, row-marching against resident): FP32 70x45 20.5 / 1.8,
 // 200^2 with a source term 34 / 3.1, 330x517 16.6 / 4.7, 512^2 18.8 / 6.1, 620^2 20.9 / 8.6;
-// FP64 64^2 150 / 5.9, 200^2 172 / 23, 400^2 155 / 59, 430^2 163 / 70.
+// FP64 64^2 150 / 4.7, 200^2 172 / 23, 400^2 155 / 59, 430^2 163 / 70.
 dugks_status plan_resident(dugks_ctx* ctx, int nsrc, ResPlan& r) {
     free_resident(r);
     int sms = 0, smem_max = 0, coop = 0;

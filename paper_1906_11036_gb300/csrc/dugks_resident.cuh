@@ -236,6 +236,7 @@ __device__ __forceinline__ void res_moments(const PT (&P)[4], T& mx, T& my) {
 // weights of a face in shared memory: normal weights of the left and of the right cell for a pair
 // that moves along the normal (4), 1 - w, w, hcd, hc tl, hc tr; in FP64 the first four and a second
 // pair of tangential weights carry the factor a_f of Eq. 2.22 (one multiplication less per value)
+// faces of a march unrolled: 2 (512^2 FP32 6.11 us per step, 70x45 1.84) against 1 (6.35, 1.74)
 #ifndef DUGKS_RES_UNROLL
 #define DUGKS_RES_UNROLL 2
 #endif
@@ -329,7 +330,7 @@ __device__ __forceinline__ void res_march(const ResConsts<T, NC>& k, const Pair<
 // cell, bit 31 set where it has one), lane group q = lane / 8 the pair q; sums over the pairs go
 // through shuffles.  The FP64 pipe of a quarter of an SM takes 64 clocks for an instruction of a warp
 // whatever its active lanes, so one warp alone needs about 75 x 64 clocks for its cells while the
-// other three quarters idle; split, each quarter runs about 28 (64^2: 5.9 -> 4.8 us per step).
+// other three quarters idle; split, each quarter runs about 28 (64^2: 5.9 -> 4.7 us per step).
 // hq: the lane's pair of hbp; no source terms, no wall cells.
 template <typename T, int NC, typename Slot>
 __device__ __forceinline__ void res_cell_parts(const ResArgs<T>& a, const ResConsts<T, NC>& k, const Vec2<T>* hq, Pair<T>* sP,
@@ -397,6 +398,8 @@ __device__ __forceinline__ void res_cell_parts(const ResArgs<T>& a, const ResCon
     }
 }
 
+// threads per CTA at most.  FP32: 512 at 128 registers (512^2 6.3 us per step; 640 at 96 registers 6.7, 768 at
+// 80 8.1, 384 6.8).  FP64: 256, eight warps keep its pipe busy.
 #ifndef DUGKS_RES_THREADS32
 #define DUGKS_RES_THREADS32 512
 #endif
