@@ -1288,12 +1288,12 @@ cudaError_t launch_adjoint_step(dugks_ctx* ctx, const void* f, long long f_pitch
         }
     }
     const int tb = adj_tile_blocks(ctx);
-    ctx->adj_used = adj_partials(ctx);
+    const int wb = adj_wall_blocks(ctx);
+    ctx->adj_used = tb + wb;  // the slots these launches write
     const size_t smem = AdjTile<T, kAdjTX, kAdjTY>::bytes();
     cudaError_t e = cudaFuncSetAttribute(adj_tile_kernel<T, NC, kAdjTX, kAdjTY>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
-    const int wb = adj_wall_blocks(ctx);
     adj_tile_kernel<T, NC, kAdjTX, kAdjTY><<<adj_tile_grid(ctx), kAdjTX * kAdjTY, smem, ctx->stream>>>(a, k, ka, g,
                                                                                                      wb > 0 ? 1 : 0);
     if (wb > 0) adj_wall_kernel<T, NC><<<wb, kAdjThreads, 0, ctx->stream>>>(a, k, ka, g, tb);
