@@ -45,6 +45,11 @@ struct AdjArgs {
     long long f_pitch, f_plane;
     const T* mu;       // dJ/d ftilde^{n+1}
     T* lam;            // out: dJ/d ftilde^n
+    // 1: mu and lam hold velocity 0 and the others' deviations from it.  mu is nearly the same for all
+    // velocities (the first one of a reverse sweep exactly), while dJ/du and the relaxation see the
+    // differences alone: kept as deviations through the sweep they do not lose their digits to lam_0
+    // (dJ/du in FP32 is off by 1e-7 where rounding lam_i itself left 3e-6 ... 2e-5).  0: as they are.
+    int dev;
     T* Ax;             // x-face adjoints [Q][ny][nx+1]
     T* Ay;             // y-face adjoints [Q][ny+1][nx]
     double* partial;   // per-block partial sums: dJ/dlambda at [slot], dJ/du_x at [pstride + slot],
@@ -99,31 +104,35 @@ __device__ __forceinline__ T poly_nc(const T (&c)[NC], T x) {
     return s;
 }
 
-// sum_i w_i d feq_i / d u_a at phi for a = x, y, over the velocities in `mask`
-// (bit i: velocity i), added to du[0], du[1] in double.  Over all velocities (kAllQ) the rest
-// velocity follows the zeroth moment, its derivative minus the sum of the others: w_i - w_0 weighs
-// the others.  w is nearly the same for all velocities there, and the rounded Au, Bu do not sum to
-// zero, which biased the derivative by up to 1e-5 in FP32.
+// sum_i w_i d feq_i / d u_a at phi for a = x, y, over the moving velocities in `mask`
+// (bit i: velocity i), added to du[0], du[1] in double.  Over all velocities pass w_i - w_0: the rest
+// velocity follows the zeroth moment, its derivative minus the sum of the others.  (w_i is nearly the
+// same for all velocities there, and the rounded Au, Bu do not sum to zero: 1e-5 of dJ/du in FP32.)
 template <typename T, int NC>
 __device__ __forceinline__ void add_du(const AdjConsts<T, NC>& ka, T phi, const T (&w)[Q], unsigned mask,
                                        double (&du)[2]) {
     const T bv = poly_nc<T, NC>(ka.bpoly, phi), cv = poly_nc<T, NC>(ka.cpoly, phi);
-    const T w0 = (mask & 1u) ? w[0] : T(0);
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
         T sa = T(0), sb = T(0);
 #pragma unroll
         for (int i = 1; i < Q; ++i)
             if (mask & (1u << i)) {
-                sa = fma(w[i] - w0, ka.Au[a][i], sa);
-                sb = fma(w[i] - w0, ka.Bu[a][i], sb);
+                sa = fma(w[i], ka.Au[a][i], sa);
+                sb = fma(w[i], ka.Bu[a][i], sb);
             }
         du[a] += double(fma(bv, sa, cv * sb));
     }
 }
 __host__ __device__ constexpr unsigned xmask() { return (1u << 1) | (1u << 3) | (1u << 5) | (1u << 6) | (1u << 7) | (1u << 8); }
 __host__ __device__ constexpr unsigned ymask() { return (1u << 2) | (1u << 4) | (1u << 5) | (1u << 6) | (1u << 7) | (1u << 8); }
-constexpr unsigned kAllQ = (1u << Q) - 1u;
+constexpr unsigned kAllQ = (1u << Q) - 2u;  // every moving velocity
+
+// a x - b y with both products rounded: the same product enters the two faces of a cell, so the
+// roundings cancel in the sums over cells (contracted to one fma they leave a bias: 0.4f x rounds to
+// 2/5 x rather than to 0.4f x on average, 6e-6 of dJ/du at 512^2)
+__device__ __forceinline__ float diff_rn(float a, float x, float b, float y) { return __fsub_rn(__fmul_rn(a, x), __fmul_rn(b, y)); }
+__device__ __forceinline__ double diff_rn(double a, double x, double b, double y) { return __dsub_rn(__dmul_rn(a, x), __dmul_rn(b, y)); }
 
 // The block's sums of v[0..2] (dJ/dlambda, dJ/du_x, dJ/du_y) into out[0], out[stride],
 // out[2 stride] (one slot per block: no race), added to the slots or overwriting them.
@@ -189,14 +198,17 @@ __global__ void __launch_bounds__(128) adj_wall_kernel(const StepArgs<T, NC> a, 
         }
         feq_all(k, phi, fe);
         dfeq_all(ka, phi, dfe);
-        T dphibar = T(0);
-        auto fold = [&](const T (&Pg)[Q], T bv) {
+        // PG: the ghosts' adjoints, those of the moving velocities as deviations from the rest velocity's
+        T add0 = T(0);
+        auto fold = [&](T (&Pg)[Q], T bv) {
             T dg[Q];
             dfeq_all(ka, T(2) * bv - phi, dg);
+            PG[0] += Pg[0];
 #pragma unroll
-            for (int i = 0; i < Q; ++i) {
+            for (int i = 1; i < Q; ++i) {
+                Pg[i] -= Pg[0];
                 PG[i] += Pg[i];
-                dphibar -= Pg[i] * (dg[i] + dfe[i]);
+                add0 -= Pg[i] * dg[i];
             }
             if (g.want_u) add_du(ka, T(2) * bv - phi, Pg, kAllQ, du);  // feq(phi_g) of the ghost
         };
@@ -244,22 +256,21 @@ __global__ void __launch_bounds__(128) adj_wall_kernel(const StepArgs<T, NC> a, 
             }
             fold(Pg, k.bcv[3]);
         }
-        // the ghosts' share of Eq. 2.21's transpose (P enters through a_bp f + b_bp feq(phi))
-        T s = T(0);
+        // the ghosts' share of Eq. 2.21's transpose (P enters through a_bp f + b_bp feq(phi)); of PG[0]
+        // itself the weights a_bp + (b_bp - 1) - 1 remain
+        T s = T(0), w[Q];
+        add0 -= PG[0];
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            dphibar += ka.b_bp * PG[i] * dfe[i];
+        for (int i = 1; i < Q; ++i) {
+            w[i] = (ka.b_bp - T(1)) * PG[i];
+            add0 += w[i] * dfe[i];
             s += PG[i] * fma(ka.da_bp, ft[i], ka.db_bp * fe[i]);
         }
         djdl = double(s);
-        if (g.want_u) {  // - feq(phi) of every ghost and b_bp feq(phi) of Eq. 2.21 through P of the cell
-            T w[Q];
+        if (g.want_u) add_du(ka, phi, w, kAllQ, du);  // - feq(phi) of every ghost, b_bp feq(phi) of Eq. 2.21 through P
+        g.lam[c] += add0;
 #pragma unroll
-            for (int i = 0; i < Q; ++i) w[i] = (ka.b_bp - T(1)) * PG[i];
-            add_du(ka, phi, w, kAllQ, du);
-        }
-#pragma unroll
-        for (int i = 0; i < Q; ++i) g.lam[i * cplane + c] += fma(ka.a_bp, PG[i], dphibar);
+        for (int i = 1; i < Q; ++i) g.lam[i * cplane + c] += fma(ka.a_bp, PG[i], g.dev ? T(0) : add0);
     }
     const double v[3] = {djdl, du[0], du[1]};
     block_partial3(v, g.partial + first_partial + blockIdx.x, g.pstride, g.accumulate);
@@ -352,7 +363,10 @@ __global__ void __launch_bounds__(TX * TY) adj_tile_kernel(const StepArgs<T, NC>
         const bool real = X.state == 0 && Y.state == 0;
         const long long c = (long long)Y.i * nx + X.i;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) sMu[(i * L::MH + mr) * L::MW + mc] = real ? g.mu[i * cplane + c] : T(0);
+        for (int i = 0; i < Q; ++i) {
+            const T m0 = real && i > 0 && !g.dev ? g.mu[c] : T(0);  // deviations from velocity 0
+            sMu[(i * L::MH + mr) * L::MW + mc] = real ? g.mu[i * cplane + c] - m0 : T(0);
+        }
     }
     __syncthreads();
 
@@ -395,10 +409,11 @@ __global__ void __launch_bounds__(TX * TY) adj_tile_kernel(const StepArgs<T, NC>
             const T rL = lghost ? T(0) : a.cx[Lc.i + 1].r, rR = rghost ? T(0) : a.cx[Rc.i + 1].r;
             T gv[Q];
             T sg = T(0);
+            const T gz = diff_rn(rR, Mt(0, xr, xc + 1), rL, Mt(0, xr, xc));
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 T v = T(0);
-                if (EX(i) != 0) v = T(EX(i)) * (rR * Mt(i, xr, xc + 1) - rL * Mt(i, xr, xc));
+                if (EX(i) != 0) v = T(EX(i)) * (gz + (rR * Mt(i, xr, xc + 1) - rL * Mt(i, xr, xc)));
                 gv[i] = v;
                 if (EX(i) != 0) sg += v * dfe[i];
             }
@@ -463,10 +478,11 @@ __global__ void __launch_bounds__(TX * TY) adj_tile_kernel(const StepArgs<T, NC>
             const T rL = lghost ? T(0) : a.cy[Lr.i + 1].r, rR = rghost ? T(0) : a.cy[Rr.i + 1].r;
             T gv[Q];
             T sg = T(0);
+            const T gz = diff_rn(rR, Mt(0, yr + 1, yc), rL, Mt(0, yr, yc));
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 T v = T(0);
-                if (EY(i) != 0) v = T(EY(i)) * (rR * Mt(i, yr + 1, yc) - rL * Mt(i, yr, yc));
+                if (EY(i) != 0) v = T(EY(i)) * (gz + (rR * Mt(i, yr + 1, yc) - rL * Mt(i, yr, yc)));
                 gv[i] = v;
                 if (EY(i) != 0) sg += v * dfe[i];
             }
@@ -538,21 +554,21 @@ __global__ void __launch_bounds__(TX * TY) adj_tile_kernel(const StepArgs<T, NC>
         }
         feq_all(k, phi, fe);
         dfeq_all(ka, phi, dfe);
-        T phibar = T(0), s = T(0);
+        // the moving velocities over the rest velocity (mu already is): the weights of Pb[0] and of mu[0]
+        // sum to one over Eqs. 2.21 and 2.13 and the equilibria, so lam_0 takes them whole
+        T l0 = Pb[0] + mu[0], s = T(0), w[Q];
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            phibar += (ka.b_bp * Pb[i] + ka.b_tp * mu[i]) * dfe[i];
+        for (int i = 1; i < Q; ++i) {
+            Pb[i] -= Pb[0];
+            w[i] = fma(ka.b_bp, Pb[i], ka.b_tp * mu[i]);
+            l0 = fma(w[i], dfe[i], l0);
             s += Pb[i] * fma(ka.da_bp, ft[i], ka.db_bp * fe[i]) + mu[i] * fma(ka.da_tp, ft[i], ka.db_tp * fe[i]);
         }
         djdl += double(s);
-        if (g.want_u) {  // Eqs. 2.21 and 2.13: b_bp feq(phi) in P and b_tp feq(phi) in ftilde^+
-            T w[Q];
+        if (g.want_u) add_du(ka, phi, w, kAllQ, du);  // Eqs. 2.21 and 2.13: b_bp feq(phi) in P and b_tp feq(phi) in ftilde^+
+        g.lam[t] = l0;
 #pragma unroll
-            for (int i = 0; i < Q; ++i) w[i] = fma(ka.b_bp, Pb[i], ka.b_tp * mu[i]);
-            add_du(ka, phi, w, kAllQ, du);
-        }
-#pragma unroll
-        for (int i = 0; i < Q; ++i) g.lam[i * cplane + t] = fma(ka.a_bp, Pb[i], fma(ka.a_tp, mu[i], phibar));
+        for (int i = 1; i < Q; ++i) g.lam[i * cplane + t] = fma(ka.a_bp, Pb[i], ka.a_tp * mu[i]) + (g.dev ? T(0) : l0);
     }
     const double v[3] = {djdl, du[0], du[1]};
     block_partial3(v, g.partial + blockIdx.y * gridDim.x + blockIdx.x, g.pstride, g.accumulate);
@@ -583,17 +599,18 @@ __global__ void __launch_bounds__(1024) adj_sum_kernel(const double* __restrict_
     }
 }
 
-// lam_i = g (the same for every velocity: phi = sum_i f_i)
+// lam_i = g (the same for every velocity: phi = sum_i f_i), as lam_0 and deviations from it
 template <typename T>
 __global__ void broadcast_phi_adjoint(const T* __restrict__ gphi, T* __restrict__ lam, long long n) {
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const T v = gphi[c];
+        lam[c] = gphi[c];
 #pragma unroll
-        for (int i = 0; i < Q; ++i) lam[i * n + c] = v;
+        for (int i = 1; i < Q; ++i) lam[i * n + c] = T(0);
     }
 }
 
-// dJ/dphi0 = sum_i feq_i'(phi0) lam_i (f^0 = feq(phi0), opening of Section 4); with upart set
+// dJ/dphi0 = sum_i feq_i'(phi0) lam_i (f^0 = feq(phi0), opening of Section 4), lam as lam_0 and
+// deviations from it (sum_i feq_i' = 1); with upart set
 // (3 gridDim.x doubles), the block's sums of sum_i lam_i d feq_i / d u_a(phi0) (f^0 depends on
 // u too) go to upart[gridDim.x + blockIdx.x] and upart[2 gridDim.x + blockIdx.x], and 0 to
 // upart[blockIdx.x].
@@ -607,10 +624,11 @@ __global__ void __launch_bounds__(256) init_adjoint_kernel(const T* __restrict__
         dfeq_all(ka, phi0[c], d);
         T s = T(0);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
+        for (int i = 1; i < Q; ++i) {
             l[i] = lam[i * n + c];
             s = fma(d[i], l[i], s);
         }
+        s += lam[c];
         gphi0[c] = s;
         if (upart) add_du(ka, phi0[c], l, kAllQ, du);
     }

@@ -58,7 +58,10 @@ struct AdjConstsP {
     float2 dq[4][NC];           // (feq_PA', feq_PB') (the top coefficient is zero)
     float2 Au[2][4], Bu[2][4];  // d feq / d u_a = Au b(phi) + Bu Cint(phi) per pair (u of B = u b)
     float bpoly[NC], cpoly[NC];
-    float a_bp, b_bp, a_tp, b_tp, a_f, b_f;
+    float a_bp, b_bp, a_tp, a_f, b_f;  // the forward step's (b_bp: 1 - a_bp)
+    // b of Eqs. 2.21 and 2.13 rounded directly: what the adjoint multiplies by them is linear in b, and
+    // 1 - a is off by up to half an ulp of one (3e-6 of b at b = 0.007)
+    float wb_bp, wb_tp;
     // d/dlambda of the weights of f, over b_bp.  Those of feq are the opposite (the weights of each of
     // Eqs. 2.13, 2.21, 2.22 sum to one), so each enters as da (f - feq), here da / b_bp times
     // b_bp f - hbp(phi): feq as the forward step rounds it, so the small difference has no bias
@@ -142,35 +145,25 @@ __device__ __forceinline__ float ap_ghost(const AdjConstsP<NC>& k, const float p
 
 // The adjoint B of such a ghost folded back into its interior cell (ftilde ft): v = the
 // addition to lam of the cell (transposes of Eq. 2.21 and of phi = sum f through both
-// equilibria); its dJ/dlambda and dJ/du terms are added to rl, ru.
+// equilibria), in the form lam is kept in: v.z to lam_0, v.p to the deviations from it; its
+// dJ/dlambda and dJ/du terms are added to rl, ru.
 template <int NC, bool WU>
 __device__ __forceinline__ void ap_ghost_fold(const AdjConstsP<NC>& k, const V9& B, const V9& ft, const float bv,
                                               V9& v, float& rl, float (&ru)[2]) {
     const float phc = vsum(ft), phg = 2.f * bv - phc;
     const F2 xc = f2(phc), xg = f2(phg);
-    const F2 c1 = f2(k.b_bp - 1.f);
-    F2 pb = f2(0.f), dcs = f2(0.f), dgs = f2(0.f), ncs = f2(0.f), sp = f2(0.f);
+    const F2 c1 = f2(k.wb_bp - 1.f);
+    F2 w[4], pb = f2(0.f), sp = f2(0.f);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const F2 dc = ap_dfeq(k, q, xc), dg = ap_dfeq(k, q, xg), nc = ap_neq(k, q, ft.p[q], xc);
-        pb = fma2(B.p[q], fma2(c1, dc, f2(-1.f) * dg), pb);
-        dcs = dcs + dc;
-        dgs = dgs + dg;
-        ncs = ncs + nc;
-        sp = fma2(B.p[q], nc, sp);
+        w[q] = B.p[q] - f2(B.z);
+        pb = fma2(w[q], fma2(c1, ap_dfeq(k, q, xc), f2(-1.f) * ap_dfeq(k, q, xg)), pb);
+        sp = fma2(w[q], ap_neq(k, q, ft.p[q], xc), sp);
+        v.p[q] = f2(k.a_bp) * w[q];
     }
-    // the rest velocity's derivatives and equilibrium follow the zeroth moment
-    const float dc0 = 1.f - hsum(dcs), dg0 = 1.f - hsum(dgs), nc0 = -hsum(ncs);
-    const float phibar = fmaf(B.z, fmaf(k.b_bp - 1.f, dc0, -dg0), hsum(pb));
-    const F2 ph2 = f2(phibar);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) v.p[q] = fma2(f2(k.a_bp), B.p[q], ph2);
-    v.z = fmaf(k.a_bp, B.z, phibar);
-    rl = fmaf(k.da_bp, fmaf(B.z, nc0, hsum(sp)), rl);
+    v.z = hsum(pb) - B.z;  // (the weights a_bp + (b_bp - 1) - 1 of B.z itself)
+    rl = fmaf(k.da_bp, hsum(sp), rl);
     if (WU) {  // (b_bp - 1) feq(phi_c) and feq(phi_g) in P_g
-        F2 w[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) w[q] = B.p[q] - f2(B.z);
         ap_add_du(k, phg, w, 0xFu, ru);
 #pragma unroll
         for (int q = 0; q < 4; ++q) w[q] = c1 * w[q];
@@ -213,8 +206,9 @@ __host__ __device__ inline void adj_region_tile(const AdjRegion& r, int b, int& 
 
 // S: ring stages (a power of two keeps the stage index a mask); WU: also form the u-derivative;
 // WALL: the grid has a Dirichlet wall on some axis (mirrored NEE ghosts, their adjoints folded
-// back into the cells they mirror; else both axes are periodic)
-template <int NC, int S, bool WU, bool WALL>
+// back into the cells they mirror; else both axes are periodic); DEV: mu and lam as velocity 0 and
+// deviations from it (AdjArgs::dev; as a branch instead it cost 1 ... 2 % of a step)
+template <int NC, int S, bool WU, bool WALL, bool DEV>
 __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUGKS_ADJ_ROWS_MIN_WARPS)
     adj_rows_kernel(const __grid_constant__ CUtensorMap tf, const __grid_constant__ CUtensorMap tmu,
                     const StepArgs<float, NC> a, const AdjConstsP<NC> k, const AdjArgs<float> g,
@@ -273,7 +267,8 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
     };
     if (lane == 0)
         for (int t = 0; t < min(S, R); ++t) issue(t);
-    // row r's ftilde (which = 0) or mu (1) as pairs: stage of row r, or the periodic image in global memory
+    // row r's ftilde (which = 0) or mu (1: mu_0 and the deviations from it) as pairs: stage of row r, or
+    // the periodic image in global memory
     auto row_v9 = [&](int r, int which, V9& v) {
         const int t = r - (y0 - 2);
         if (from_smem) {
@@ -293,6 +288,9 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
 #pragma unroll
             for (int q = 0; q < 4; ++q) v.p[q] = f2(src[PA(q) * pl], src[PB(q) * pl]);
         }
+        if (!DEV && which)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v.p[q] = v.p[q] - f2(v.z);
     };
 
     V9 Pm2, Pm1, Pn;  // P = fbar^+ of rows n-2, n-1, n (this lane's column)
@@ -380,11 +378,12 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
             }
             // adjoint of the face's f (Eq. 2.12 flux): e_x (r_R mu_R - r_L mu_L)
             F2 gv[3];
+            const float zr = __fmul_rn(mq.z, cxj.r), gz = __shfl_down_sync(0xffffffffu, zr, 1) - zr;
 #pragma unroll
             for (int s = 0; s < 3; ++s) {
                 const int q = s == 0 ? 0 : s + 1;
                 const F2 rm = mq.p[q] * f2(float(QX(q)) * cxj.r, -float(QX(q)) * cxj.r);
-                gv[s] = shfl_dn2(rm) - rm;
+                gv[s] = (shfl_dn2(rm) - rm) + f2(float(QX(q)) * gz, -float(QX(q)) * gz);
             }
             // Eq. 2.22 transposed: A = a_f gv + b_f sum_m gv_m feq_m'(phi_b)
             const F2 pb2 = f2(phib);
@@ -446,6 +445,7 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
             V9 mn;
             row_v9(n, 1, mn);
             F2 fb[3], gv[3];
+            const float gz = __fsub_rn(__fmul_rn(mn.z, rR), __fmul_rn(mq.z, rL));
 #pragma unroll
             for (int s = 0; s < 3; ++s) {
                 const int q = s + 1;
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
                     v = fma2(f2(-float(QX(q)) * k.hc, float(QX(q)) * k.hc), gt, v);
                 }
                 fb[s] = v;
-                gv[s] = fma2(mn.p[q], f2(rR, -rR), mq.p[q] * f2(-rL, rL));  // e_y (r_R mu_R - r_L mu_L)
+                gv[s] = fma2(mn.p[q], f2(rR, -rR), fma2(mq.p[q], f2(-rL, rL), f2(gz, -gz)));  // e_y (r_R mu_R - r_L mu_L)
             }
             const float phib = fmaf(1.f - m.w, ph1,
                                     fmaf(m.w, phn, fmaf(m.hcd, my1 - myn, -k.hc * fmaf(m.tl, gmx1, m.tr * gmxn))));
@@ -534,20 +534,17 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
             row_v9(r, 1, mu);
             const float phi = vsum(ft);
             const F2 x2 = f2(phi);
-            F2 w[4];
-            F2 pb = f2(0.f), dsum = f2(0.f), nsum = f2(0.f), sp = f2(0.f);
+            F2 w[4], dl[4];  // (velocities over the rest velocity: its own weights sum to one)
+            F2 pb = f2(0.f), sp = f2(0.f);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const F2 de = ap_dfeq(k, q, x2), ne = ap_neq(k, q, ft.p[q], x2);
-                w[q] = fma2(f2(k.b_bp), Ba.p[q], f2(k.b_tp) * mu.p[q]);
-                pb = fma2(w[q], de, pb);
-                dsum = dsum + de;
-                nsum = nsum + ne;
-                sp = fma2(fma2(f2(k.da_bp), Ba.p[q], f2(k.da_tp) * mu.p[q]), ne, sp);
+                const F2 v = Ba.p[q] - f2(Ba.z);
+                w[q] = fma2(f2(k.wb_bp), v, f2(k.wb_tp) * mu.p[q]);
+                pb = fma2(w[q], ap_dfeq(k, q, x2), pb);
+                sp = fma2(fma2(f2(k.da_bp), v, f2(k.da_tp) * mu.p[q]), ap_neq(k, q, ft.p[q], x2), sp);
+                dl[q] = fma2(f2(k.a_bp), v, f2(k.a_tp) * mu.p[q]);
             }
-            const float de0 = 1.f - hsum(dsum), ne0 = -hsum(nsum);  // rest velocity: zeroth moment
-            const float wz = fmaf(k.b_bp, Ba.z, k.b_tp * mu.z);
-            const float phibar = fmaf(wz, de0, hsum(pb));
+            const float lz = (Ba.z + mu.z) + hsum(pb);
             V9 addv;  // folds of the mirrored ghosts of this cell (walls)
 #pragma unroll
             for (int q = 0; q < 4; ++q) addv.p[q] = f2(0.f);
@@ -590,12 +587,8 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
                 }
             }
             if (owner) {
-                rl += fmaf(fmaf(k.da_bp, Ba.z, k.da_tp * mu.z), ne0, hsum(sp));
-                if (WU) {  // b_bp feq(phi) in P, b_tp feq(phi) in ftilde^+
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) w[q] = w[q] - f2(wz);
-                    ap_add_du(k, phi, w, 0xFu, ru);
-                }
+                rl += hsum(sp);
+                if (WU) ap_add_du(k, phi, w, 0xFu, ru);  // b_bp feq(phi) in P, b_tp feq(phi) in ftilde^+
                 if constexpr (WALL) {
                     rl += addl;
                     if (WU) {
@@ -603,14 +596,17 @@ __global__ void __launch_bounds__(32, WALL ? DUGKS_ADJ_ROWS_WALL_MIN_WARPS : DUG
                         ru[1] += addu[1];
                     }
                 }
-                const F2 ph2 = f2(phibar);
+                const float l0 = lz + addv.z;
+                if (!DEV)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) dl[q] = dl[q] + f2(l0);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const F2 l = fma2(f2(k.a_bp), Ba.p[q], fma2(f2(k.a_tp), mu.p[q], ph2)) + addv.p[q];
+                    const F2 l = dl[q] + addv.p[q];
                     out[PA(q) * cplane] = l.v.x;
                     out[PB(q) * cplane] = l.v.y;
                 }
-                out[0] = fmaf(k.a_bp, Ba.z, fmaf(k.a_tp, mu.z, phibar)) + addv.z;
+                out[0] = l0;
             }
         }
         djdl += double(rl);

@@ -1080,7 +1080,8 @@ AdjConstsP<NC> make_adj_consts_p(const dugks_ctx* ctx) {
         p.bpoly[m] = ka.bpoly[m];
         p.cpoly[m] = ka.cpoly[m];
     }
-    p.a_bp = k.a_bp; p.b_bp = k.b_bp; p.a_tp = k.a_tp; p.b_tp = k.b_tp; p.a_f = k.a_f; p.b_f = k.b_f;  // the forward step's
+    p.a_bp = k.a_bp; p.b_bp = k.b_bp; p.a_tp = k.a_tp; p.a_f = k.a_f; p.b_f = k.b_f;
+    p.wb_bp = ka.b_bp; p.wb_tp = ka.b_tp;
     p.da_bp = float(double(ka.da_bp) / k.b_bp); p.da_tp = float(double(ka.da_tp) / k.b_bp);
     p.da_f = float(double(ka.da_f) / k.b_bp);
     p.hc = k.hc;
@@ -1227,7 +1228,8 @@ cudaError_t launch_adjoint_rows(dugks_ctx* ctx, const StepArgs<float, NC>& a, co
         at.val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = &at;
         cfg.numAttrs = overlap ? 1 : 0;
-        return cudaLaunchKernelEx(&cfg, adj_rows_kernel<NC, kAdjRowStages, WU, WALL>, tm[0], tm[1], a, kp, g, seg, r);
+        return g.dev ? cudaLaunchKernelEx(&cfg, adj_rows_kernel<NC, kAdjRowStages, WU, WALL, true>, tm[0], tm[1], a, kp, g, seg, r)
+                     : cudaLaunchKernelEx(&cfg, adj_rows_kernel<NC, kAdjRowStages, WU, WALL, false>, tm[0], tm[1], a, kp, g, seg, r);
     };
     auto pick = [&](auto wall, const AdjRegion& r, bool overlap) {
         return g.want_u ? launch(std::true_type{}, wall, r, overlap) : launch(std::false_type{}, wall, r, overlap);
@@ -1257,10 +1259,10 @@ cudaError_t launch_adjoint_rows(dugks_ctx* ctx, const StepArgs<float, NC>& a, co
 // One adjoint step.  accumulate: the step's partials are added to the partial buffer (a
 // reverse sweep zeroes it first and sums it at the end); else they overwrite it and, with
 // dj_dalpha set, are summed into *dj_dalpha (and dj_du[0..1] if set).  want_u: also form
-// the u-derivative.
+// the u-derivative.  dev: mu and lam as velocity 0 and deviations from it (AdjArgs).
 template <typename T, int NC>
 cudaError_t launch_adjoint_step(dugks_ctx* ctx, const void* f, long long f_pitch, const void* mu, void* lam,
-                                double* dj_dalpha, double* dj_du, bool want_u, bool accumulate) {
+                                double* dj_dalpha, double* dj_du, bool want_u, bool accumulate, bool dev) {
     StepArgs<T, NC> a = make_args<T, NC>(ctx, 0);
     a.fin = static_cast<const T*>(f);  // the adjoint reads contiguous [Q][ny][nx] states
     a.pitch = ctx->nx;
@@ -1273,6 +1275,7 @@ cudaError_t launch_adjoint_step(dugks_ctx* ctx, const void* f, long long f_pitch
     g.f_plane = f_pitch * ctx->ny;
     g.mu = static_cast<const T*>(mu);
     g.lam = static_cast<T*>(lam);
+    g.dev = dev ? 1 : 0;
     g.Ax = static_cast<T*>(ctx->adj_ax);
     g.Ay = static_cast<T*>(ctx->adj_ay);
     g.partial = ctx->adj_partial;
@@ -1303,19 +1306,19 @@ cudaError_t launch_adjoint_step(dugks_ctx* ctx, const void* f, long long f_pitch
 
 // f: rows f_pitch elements apart (nx: contiguous, or the pitch of the context's own states)
 cudaError_t launch_adjoint_step_any(dugks_ctx* ctx, const void* f, long long f_pitch, const void* mu, void* lam,
-                                    double* dj_dalpha, double* dj_du, bool want_u, bool accumulate) {
+                                    double* dj_dalpha, double* dj_du, bool want_u, bool accumulate, bool dev) {
     const int nc = want_u ? std::max(ctx->nc, ctx->nc_u) : ctx->nc;
     if (ctx->precision == 32) {
         switch (nc) {
-            case 3: return launch_adjoint_step<float, 3>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
-            case 4: return launch_adjoint_step<float, 4>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
-            default: return launch_adjoint_step<float, NC_LARGE>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
+            case 3: return launch_adjoint_step<float, 3>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate, dev);
+            case 4: return launch_adjoint_step<float, 4>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate, dev);
+            default: return launch_adjoint_step<float, NC_LARGE>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate, dev);
         }
     }
     switch (nc) {
-        case 3: return launch_adjoint_step<double, 3>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
-        case 4: return launch_adjoint_step<double, 4>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
-        default: return launch_adjoint_step<double, NC_LARGE>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate);
+        case 3: return launch_adjoint_step<double, 3>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate, dev);
+        case 4: return launch_adjoint_step<double, 4>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate, dev);
+        default: return launch_adjoint_step<double, NC_LARGE>(ctx, f, f_pitch, mu, lam, dj_dalpha, dj_du, want_u, accumulate, dev);
     }
 }
 
@@ -2029,7 +2032,8 @@ dugks_status dugks_adjoint_step(dugks_ctx* ctx, const void* f_dev, const void* m
     DeviceGuard guard(ctx->device);
     dugks_status st = adj_alloc(ctx);
     if (st != DUGKS_OK) return st;
-    CK(launch_adjoint_step_any(ctx, f_dev, ctx->nx, mu_dev, lam_dev, dj_dalpha_dev, dj_du_dev, dj_du_dev != nullptr, false));
+    CK(launch_adjoint_step_any(ctx, f_dev, ctx->nx, mu_dev, lam_dev, dj_dalpha_dev, dj_du_dev, dj_du_dev != nullptr, false,
+                               false));
     return DUGKS_OK;
 }
 
@@ -2137,8 +2141,8 @@ dugks_status dugks_adjoint(dugks_ctx* ctx, const void* phi0_dev, long long nstep
         if (ns > 1 && (e = advance(s, nck + ns - 1, ns - 1, true)) != cudaSuccess) return fail(e, "recomputed segment");
         for (long long q = ns - 1; q >= 0; --q) {
             const void* f = q == 0 ? state[size_t(s)] : seg[q];
-            if ((e = launch_adjoint_step_any(ctx, f, ctx->pitch, lam[cur], lam[1 - cur], nullptr, nullptr, want_u, true)) !=
-                cudaSuccess)
+            if ((e = launch_adjoint_step_any(ctx, f, ctx->pitch, lam[cur], lam[1 - cur], nullptr, nullptr, want_u, true,
+                                             true)) != cudaSuccess)
                 return fail(e, "adjoint step");
             cur ^= 1;
         }
