@@ -44,7 +44,8 @@ typedef enum {
     DUGKS_ERR_NONFINITE = 4,   /* NaN or Inf detected in phi */
     DUGKS_ERR_UNSUPPORTED = 5, /* valid request that the library does not implement */
     DUGKS_ERR_NOMEM = 6,       /* device or host allocation failed */
-    DUGKS_ERR_TIMEOUT = 7      /* a bounded device-side wait expired; the step result is invalid */
+    DUGKS_ERR_TIMEOUT = 7      /* a bounded device-side wait expired: the state is invalid (and may mix steps), every
+                                  later call that synchronises says so again; create the context anew */
 } dugks_status;
 
 enum { DUGKS_BC_PERIODIC = 0, DUGKS_BC_DIRICHLET = 1 };
@@ -180,11 +181,11 @@ dugks_status dugks_step(dugks_ctx *ctx, long long n);
  * [ny][nx], precision's element type; may be NULL) and, if mass_out is not
  * NULL, the mass M = sum |V_jk| phi_jk accumulated in double into *mass_out
  * (host).  With mass_out != NULL the call synchronises the stream and returns
- * DUGKS_ERR_NONFINITE if M is not finite. */
+ * DUGKS_ERR_TIMEOUT if a bounded wait expired, DUGKS_ERR_NONFINITE if M is not finite. */
 dugks_status dugks_get_phi(dugks_ctx *ctx, void *phi_dev_out, double *mass_out);
 
 /* Same into a HOST array of doubles [ny][nx] (phi_host_out may be NULL);
- * synchronises the stream. */
+ * synchronises the stream and reports as dugks_get_phi does. */
 dugks_status dugks_get_phi_host(dugks_ctx *ctx, double *phi_host_out, double *mass_out);
 
 /* Copy the current ftilde state out to / in from a caller device buffer laid
@@ -281,7 +282,7 @@ dugks_status dugks_set_adjoint_kernel(dugks_ctx *ctx, int kernel);
  * from the last recomputes its states and steps the adjoint back through it
  * (memory: ceil(nsteps/K) + K + 2 states of 9 nx ny elements in one workspace
  * that the context keeps for later calls, grown when a call needs more and
- * freed by dugks_destroy).  Synchronises the stream.  The context's own state
+ * freed by dugks_destroy).  Synchronises the stream; DUGKS_ERR_TIMEOUT if a bounded wait expired.  The context's own state
  * is left at an intermediate step: initialise it again before stepping. */
 dugks_status dugks_adjoint(dugks_ctx *ctx, const void *phi0_dev, long long nsteps, int checkpoint_every,
                            const void *grad_phiN_dev, void *grad_phi0_dev, double *grad_alpha_out,

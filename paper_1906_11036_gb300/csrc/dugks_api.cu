@@ -76,8 +76,11 @@ struct dugks_ctx {
     double* dyv = nullptr;
     double* staging = nullptr;  // nx*ny doubles for host transfers
     double* partial = nullptr;  // reduction partials
-    double* mass_dev = nullptr;
-    int* err_dev = nullptr;
+    // five doubles in one allocation, so that a call that reads a result back gets the error word with it
+    double* scalars = nullptr;
+    double* mass_dev = nullptr;    // scalars[0]
+    double* adj_dalpha = nullptr;  // scalars[1 .. 3]: dJ/dalpha, dJ/du_x, dJ/du_y of dugks_adjoint
+    int* err_dev = nullptr;        // in scalars[4]: bit 0 a bounded wait expired, bit 2 a negative equilibrium
     int red_blocks = 0;
     CUtensorMap tmap[2];
     int nt = 32, stages = 8, seg_rows = 0, nstrips = 0, nseg = 0, occupancy = 0;
@@ -98,7 +101,6 @@ struct dugks_ctx {
     int adj_used = 0;               // partial slots the last adjoint launch wrote (the sums read these)
     void* adj_ws = nullptr;         // dugks_adjoint's states (checkpoints, a segment, two lambdas), kept
     size_t adj_ws_bytes = 0;        //   for later calls and grown when a call needs more
-    double* adj_dalpha = nullptr;
     // source terms (dugks_set_source)
     double ux = 0, uy = 0;
     int nb = 0;
@@ -123,6 +125,7 @@ struct dugks_ctx {
     std::string last_error;
 };
 
+constexpr int kScalars = 5;              // dugks_ctx::scalars
 constexpr int kBatchShortRows = 8;       // rows of the short tiles at the end of the batched queue
 
 struct dugks_batch {
@@ -158,6 +161,23 @@ dugks_status cuda_fail(dugks_ctx* ctx, cudaError_t e, const char* what) {
         cudaError_t e_ = (call);                                  \
         if (e_ != cudaSuccess) return cuda_fail(ctx, e_, #call);  \
     } while (0)
+
+// the error word of a bounded wait -> status; such a wait leaves the state invalid for good
+dugks_status wait_status(dugks_ctx* ctx, int err) {
+    if (!(err & 1)) return DUGKS_OK;
+    ctx->last_error = "a bounded wait of a kernel expired (for a copy, or for a neighbouring tile): the state is invalid, "
+                      "create the context anew";
+    return DUGKS_ERR_TIMEOUT;
+}
+
+// synchronises and reads the scalars back, the error word among them
+dugks_status read_scalars(dugks_ctx* ctx, double (&v)[kScalars]) {
+    CK(cudaMemcpyAsync(v, ctx->scalars, sizeof(v), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    int err = 0;
+    memcpy(&err, &v[4], sizeof(err));
+    return wait_status(ctx, err);
+}
 
 bool finite_all(const double* v, int n) {
     for (int i = 0; i < n; ++i)
@@ -997,12 +1017,10 @@ void free_ctx(dugks_ctx* ctx) {
     for (void* p : {ctx->buf[0], ctx->buf[1], ctx->fxm, ctx->fym, ctx->cxm, ctx->cym, static_cast<void*>(ctx->rowy),
                     ctx->adj_ax, ctx->adj_ay,
                     ctx->src_field, ctx->hist[0], ctx->hist[1], ctx->aux[0], ctx->aux[1],
-                    static_cast<void*>(ctx->adj_partial), static_cast<void*>(ctx->adj_dalpha),
-                    static_cast<void*>(ctx->adj_upart), ctx->adj_ws})
+                    static_cast<void*>(ctx->adj_partial), static_cast<void*>(ctx->adj_upart), ctx->adj_ws})
         if (p) cudaFree(p);
     for (void* p : {static_cast<void*>(ctx->dxv), static_cast<void*>(ctx->dyv), static_cast<void*>(ctx->staging),
-                    static_cast<void*>(ctx->partial), static_cast<void*>(ctx->mass_dev),
-                    static_cast<void*>(ctx->err_dev)})
+                    static_cast<void*>(ctx->partial), static_cast<void*>(ctx->scalars)})
         if (p) cudaFree(p);
     free_resident(ctx->res);
     free_resident(ctx->res_src);
@@ -1159,7 +1177,6 @@ dugks_status adj_alloc(dugks_ctx* ctx) {
     if ((e = cudaMalloc(&ctx->adj_ax, Q * nxf * ctx->elem)) != cudaSuccess ||
         (e = cudaMalloc(&ctx->adj_ay, Q * nyf * ctx->elem)) != cudaSuccess ||
         (e = cudaMalloc(&ctx->adj_partial, 3 * sizeof(double) * size_t(adj_partials(ctx)))) != cudaSuccess ||
-        (e = cudaMalloc(&ctx->adj_dalpha, 3 * sizeof(double))) != cudaSuccess ||
         (e = cudaMalloc(&ctx->adj_upart, 3 * sizeof(double) * size_t(init_blocks(ctx)))) != cudaSuccess)
         return cuda_fail(ctx, e, "cudaMalloc(adjoint buffers)");
     return DUGKS_OK;
@@ -1688,11 +1705,13 @@ static dugks_status create_ctx(const dugks_mesh* mesh, const dugks_vset* vset, c
     if ((e = cudaMalloc(&ctx->staging, sizeof(double) * size_t(ncell))) != cudaSuccess)
         return fail(cuda_fail(ctx, e, "cudaMalloc(staging)"));
     if ((e = cudaMalloc(&ctx->partial, sizeof(double) * size_t(ctx->red_blocks))) != cudaSuccess ||
-        (e = cudaMalloc(&ctx->mass_dev, sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&ctx->err_dev, sizeof(int))) != cudaSuccess)
+        (e = cudaMalloc(&ctx->scalars, kScalars * sizeof(double))) != cudaSuccess)
         return fail(cuda_fail(ctx, e, "cudaMalloc(scalars)"));
-    if ((e = cudaMemsetAsync(ctx->err_dev, 0, sizeof(int), ctx->stream)) != cudaSuccess)
-        return fail(cuda_fail(ctx, e, "cudaMemsetAsync(err)"));
+    ctx->mass_dev = ctx->scalars;
+    ctx->adj_dalpha = ctx->scalars + 1;
+    ctx->err_dev = reinterpret_cast<int*>(ctx->scalars + 4);
+    if ((e = cudaMemsetAsync(ctx->scalars, 0, kScalars * sizeof(double), ctx->stream)) != cudaSuccess)
+        return fail(cuda_fail(ctx, e, "cudaMemsetAsync(scalars)"));
     if (ctx->kernel == DUGKS_KERNEL_FUSED) {
         st = make_state_maps(ctx, ctx->buf, 2, ctx->tmap);
         if (st != DUGKS_OK) return fail(st);
@@ -1806,10 +1825,11 @@ dugks_status dugks_get_phi(dugks_ctx* ctx, void* phi_dev_out, double* mass_out) 
     cudaError_t e = ctx->precision == 32 ? launch_phi<float, float>(ctx, static_cast<float*>(phi_dev_out))
                                          : launch_phi<double, double>(ctx, static_cast<double*>(phi_dev_out));
     CK(e);
-    CK(cudaMemcpyAsync(mass_out, ctx->mass_dev, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    if (!std::isfinite(*mass_out)) return DUGKS_ERR_NONFINITE;
-    return DUGKS_OK;
+    double v[kScalars];
+    const dugks_status st = read_scalars(ctx, v);
+    if (st != DUGKS_OK) return st;
+    *mass_out = v[0];
+    return std::isfinite(v[0]) ? DUGKS_OK : DUGKS_ERR_NONFINITE;
 }
 
 dugks_status dugks_get_phi_host(dugks_ctx* ctx, double* phi_host_out, double* mass_out) {
@@ -1821,12 +1841,11 @@ dugks_status dugks_get_phi_host(dugks_ctx* ctx, double* phi_host_out, double* ma
     const size_t n = size_t(ctx->nx) * ctx->ny;
     if (phi_host_out)
         CK(cudaMemcpyAsync(phi_host_out, ctx->staging, n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    double m = 0.0;
-    CK(cudaMemcpyAsync(&m, ctx->mass_dev, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    if (mass_out) *mass_out = m;
-    if (!std::isfinite(m)) return DUGKS_ERR_NONFINITE;
-    return DUGKS_OK;
+    double v[kScalars];
+    const dugks_status st = read_scalars(ctx, v);
+    if (st != DUGKS_OK) return st;
+    if (mass_out) *mass_out = v[0];
+    return std::isfinite(v[0]) ? DUGKS_OK : DUGKS_ERR_NONFINITE;
 }
 
 dugks_status dugks_save_state(dugks_ctx* ctx, void* f_dev_out) {
@@ -1861,10 +1880,8 @@ dugks_status dugks_sync(dugks_ctx* ctx) {
     CK(cudaStreamSynchronize(ctx->stream));
     int err = 0;
     CK(cudaMemcpy(&err, ctx->err_dev, sizeof(int), cudaMemcpyDeviceToHost));
-    if (err & 1) {
-        ctx->last_error = "a bounded TMA wait in the step kernel expired";
-        return DUGKS_ERR_TIMEOUT;
-    }
+    const dugks_status st = wait_status(ctx, err);
+    if (st != DUGKS_OK) return st;
     if (err & 4) {
         ctx->last_error = "dugks_init_phi: the equilibrium of phi0 is negative in some cell";
         return DUGKS_ERR_CONFIG;
@@ -2151,15 +2168,12 @@ dugks_status dugks_adjoint(dugks_ctx* ctx, const void* phi0_dev, long long nstep
     e = ctx->precision == 32 ? launch_init_adjoint<float>(ctx, phi0_dev, lam[cur], grad_phi0_dev, du_dev)
                              : launch_init_adjoint<double>(ctx, phi0_dev, lam[cur], grad_phi0_dev, du_dev);
     if (e != cudaSuccess) return fail(e, "init adjoint");
-    double res[3] = {0.0, 0.0, 0.0};
-    if ((e = cudaMemcpyAsync(res, ctx->adj_dalpha, 3 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream)) !=
-        cudaSuccess)
-        return fail(e, "cudaMemcpyAsync");
-    if ((e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) return fail(e, "cudaStreamSynchronize");
-    if (grad_alpha_out) *grad_alpha_out = res[0];
+    double v[kScalars];
+    if ((st = read_scalars(ctx, v)) != DUGKS_OK) return st;
+    if (grad_alpha_out) *grad_alpha_out = v[1];
     if (grad_u_out) {
-        grad_u_out[0] = res[1];
-        grad_u_out[1] = res[2];
+        grad_u_out[0] = v[2];
+        grad_u_out[1] = v[3];
     }
     return DUGKS_OK;
 }
@@ -2272,7 +2286,8 @@ dugks_status dugks_batch_step(dugks_batch* b, long long n) {
 
 dugks_status dugks_batch_get_phi(dugks_batch* b, int i, void* phi_dev_out, double* mass_out) {
     if (!b || i < 0 || i >= b->n) return DUGKS_ERR_ARG;
-    return dugks_get_phi(b->ctx[size_t(i)], phi_dev_out, mass_out);
+    const dugks_status st = dugks_get_phi(b->ctx[size_t(i)], phi_dev_out, mass_out);
+    return st == DUGKS_OK && mass_out ? dugks_batch_sync(b) : st;  // (the batch's step has an error word of its own)
 }
 
 dugks_status dugks_batch_save_state(dugks_batch* b, int i, void* f_dev_out) {
@@ -2291,7 +2306,7 @@ dugks_status dugks_batch_sync(dugks_batch* b) {
     if ((e = cudaMemcpy(&err, b->d_err, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess)
         return batch_fail(b, e, "cudaMemcpy");
     if (err) {
-        b->last_error = "a bounded TMA wait in the batched step expired";
+        b->last_error = "a bounded wait in the batched step expired: the states are invalid, create the batch anew";
         return DUGKS_ERR_TIMEOUT;
     }
     return DUGKS_OK;
