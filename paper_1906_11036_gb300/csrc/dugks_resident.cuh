@@ -35,8 +35,10 @@
 // read it.  The step number comes from a counter of the CTA in device memory,
 // so a launch replayed from a CUDA graph does not meet its own old words.
 // All CTAs of a launch must run at once: the launch is cooperative.  Every
-// wait is bounded (2 s); a wait that expires sets the error word and ends the
-// launch without writing the state.
+// wait is bounded; one that expires sets the error word, which ends every tile
+// that waits after that.  Tiles out of its reach may still finish and store
+// their cells: the state is then invalid, the step counters differ, and later
+// launches return at once.
 //
 // In FP32 the arithmetic is that of sv_rows operation by operation: a grid
 // gives the same bits whether it runs here, in step_vp or in a batch.

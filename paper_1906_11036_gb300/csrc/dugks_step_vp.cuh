@@ -115,9 +115,10 @@ __device__ __forceinline__ void sv_ghost(const ConstsP<NC>& k, SvCell& c, const 
 // the routine (several inlined copies in one loop exhaust the register budget).  PLAIN: a
 // warp that meets neither (known at compile time), so the flags and their branches fold away.
 // `ring` counts the rows this warp already passed through its ring (row t of the warp
-// uses stage t % S in phase (t / S) & 1), so a warp may run several segments.
+// uses stage t % S in phase (t / S) & 1), so a warp may run several segments.  False if a bounded wait
+// expired: rows are then missing, and the error word is set.
 template <int NC, bool PLAIN = false>
-__device__ __forceinline__ void sv_rows(const CUtensorMap* tin, const StepArgs<float, NC>& a, const ConstsP<NC>& k,
+__device__ __forceinline__ bool sv_rows(const CUtensorMap* tin, const StepArgs<float, NC>& a, const ConstsP<NC>& k,
                                         const RowY* __restrict__ rw, unsigned char* stages, uint64_t* bars,
                                         const int S, const int lane, const int xw, const int y0, const int y1,
                                         const bool edge_in, const bool yg_in, int& ring) {
@@ -356,6 +357,7 @@ __device__ __forceinline__ void sv_rows(const CUtensorMap* tin, const StepArgs<f
     }
     ring += issued;
     __syncwarp();
+    return !failed;
 }
 
 // resident warps per SM the step kernel is compiled for (its register budget)
@@ -429,7 +431,8 @@ __global__ void __launch_bounds__(32, DUGKS_SV_MIN_WARPS)
 // visible (fence) before its count rises, and the tile that reads the count orders its TMA loads,
 // which run in the asynchronous proxy, after it.  A tile overwrites the state of two steps before
 // only after its neighbours have counted the step that read it.  Waits are bounded; one that expires
-// sets the error word, which ends the CTAs that follow at once.  us per step, a launch per step ->
+// sets the error word and the counter's top bit, and every CTA that takes a tile or waits after that
+// ends.  us per step, a launch per step ->
 // flow_vp: 1024^2 periodic 25.8 -> 21.2, 2048^2 periodic 76.1 -> 64, 2048^2 tanh mesh 64.4 -> 60.9,
 // 1500x900 with walls 32.0 -> 24.0, 800x700 20.6 -> 16.4.  (CTAs that stay and take their next tile
 // ahead of time were slower, 31 us at 1024^2: a tile taken ahead holds up its neighbours.)
@@ -437,6 +440,7 @@ struct FlowPlan {
     int rows, nseg, nstrips;
     unsigned* sync;  // [0]: tiles taken; [1 + tile]: steps done (all zero at launch)
 };
+constexpr unsigned kFlowFailed = 0x80000000u;  // in sync[0] (a launch has fewer tiles): a wait expired
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -468,7 +472,8 @@ __global__ void __launch_bounds__(32, DUGKS_SV_MIN_WARPS)
     const unsigned step = t / tiles, tile = t - step * tiles;
     const int sg = int(tile / unsigned(fp.nstrips)), st = int(tile) - sg * fp.nstrips;
     const int xw = st * L::WI, y0 = sg * fp.rows, y1 = min(y0 + fp.rows, a0.ny);
-    bool ok = true;
+    if (t & kFlowFailed) return;
+    bool ok = step > 0 || !(*reinterpret_cast<volatile int*>(a0.err) & 1);  // (a wait of an earlier launch)
     if (step > 0 && lane < 9) {
         int ns = st + lane % 3 - 1, ng = sg + lane / 3 - 1;
         bool need = true;
@@ -496,7 +501,10 @@ __global__ void __launch_bounds__(32, DUGKS_SV_MIN_WARPS)
         }
     }
     if (__any_sync(0xffffffffu, !ok)) {
-        if (lane == 0) atomicOr(a0.err, 1);
+        if (lane == 0) {
+            atomicOr(a0.err, 1);
+            atomicOr(fp.sync, kFlowFailed);
+        }
         return;  // (no copy is in flight yet)
     }
     asm volatile("fence.proxy.async;" ::: "memory");
@@ -511,11 +519,14 @@ __global__ void __launch_bounds__(32, DUGKS_SV_MIN_WARPS)
     const bool yg = !a.yper && (y0 == 0 || y1 == a.ny);
     int ring = 0;
     if (IP && !edge && !yg)
-        sv_rows<NC, true>(tin, a, k, rw, smem, bars, S, lane, xw, y0, y1, false, false, ring);
+        ok = sv_rows<NC, true>(tin, a, k, rw, smem, bars, S, lane, xw, y0, y1, false, false, ring);
     else
-        sv_rows<NC>(tin, a, k, rw, smem, bars, S, lane, xw, y0, y1, edge, yg, ring);
-    __syncwarp();  // every lane's stores come before the count
-    if (lane == 0) st_release(fp.sync + 1 + tile, step + 1u);
+        ok = sv_rows<NC>(tin, a, k, rw, smem, bars, S, lane, xw, y0, y1, edge, yg, ring);
+    __syncwarp();  // every lane's stores come before the count; a tile with rows missing is not counted
+    if (lane == 0) {
+        if (ok) st_release(fp.sync + 1 + tile, step + 1u);
+        else atomicOr(fp.sync, kFlowFailed);
+    }
 }
 
 // ---------------------------------------------------------------------------

@@ -38,3 +38,24 @@ def test_results_after_an_expired_wait(call, prec):
             calls[call]()
         assert ei.value.status == 7
     s.close()
+
+
+@pytest.mark.parametrize("nx,ny,prec", [(40, 30, 32), (40, 30, 64), (900, 700, 32)])
+def test_many_step_launches_after_an_expired_wait_leave_the_state(nx, ny, prec):
+    """The kernels that take many steps per launch end at once where the error word is set already: they
+    neither advance the state nor count steps that other tiles would take as done."""
+    from paper_1906_11036_gb300.dugks import DugksError, Solver
+
+    p, phi0 = I.burgers(nx, ny)
+    s = Solver(p, precision=prec)
+    s.init_phi(torch.tensor(phi0, device="cuda"))
+    s.step(4)
+    before = s.save_state()
+    s.wait_timeout_check(2000)
+    s.step(6)
+    after = s.save_state()
+    with pytest.raises(DugksError) as ei:
+        s.sync()
+    assert ei.value.status == 7
+    assert torch.equal(before, after)
+    s.close()
