@@ -211,6 +211,15 @@ dugks_status dugks_sync(dugks_ctx *ctx);
  * DUGKS_ERR_ARG for a null ctx or a limit outside the range. */
 dugks_status dugks_wait_timeout_check(dugks_ctx *ctx, int limit_us);
 
+/* The same for the waits between the tiles of the kernels that take many steps
+ * per launch: launches two steps in which one tile's messages (or its step
+ * count) never come and every such wait ends after limit_us microseconds.  The
+ * launch gives up, the next dugks_sync returns DUGKS_ERR_TIMEOUT, and the
+ * context has to be created anew.  DUGKS_ERR_ARG as above;
+ * DUGKS_ERR_UNSUPPORTED where no tiles wait for one another (one tile, or a
+ * launch per step). */
+dugks_status dugks_tile_timeout_check(dugks_ctx *ctx, int limit_us);
+
 /* Sizes and launch shape of a context. */
 dugks_status dugks_info(const dugks_ctx *ctx, dugks_info_t *out);
 

@@ -40,10 +40,13 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 
 }  // namespace
 
+constexpr unsigned long long kWaitNs = 2000000000ull;  // limit of a tile's wait for its neighbours
+
 // tiles of the resident step (dugks_resident.cuh); ntx = 0: the grid does not take it
 struct ResPlan {
     int ntx = 0, nty = 0, txm = 0, tym = 0, seq = 0, march = 1, threads = 0;
     size_t smem = 0;
+    unsigned long long wait_ns = kWaitNs;
     uint4* xch = nullptr;       // published cells
     unsigned* epoch = nullptr;  // steps done per tile, behind them
     bool owned = false;         // xch is an allocation of its own
@@ -90,7 +93,7 @@ struct dugks_ctx {
     int nseg_sp_src = 0;
     SegPlan sp{1, 0, 1};  // step_vp: long segments first, then short ones
     ResPlan res, res_src;  // the resident step without and with source terms
-    FlowPlan flow{0, 0, 0, nullptr};  // flow_vp (rows = 0: not taken)
+    FlowPlan flow{0, 0, 0, nullptr, kWaitNs};  // flow_vp (rows = 0: not taken)
     bool flow_plain = false;          // with the interior variant
     long long steps_done = 0;
     // adjoint work buffers (allocated on first use)
@@ -816,6 +819,7 @@ cudaError_t launch_resident(dugks_ctx* ctx, int n, const void* in, void* out, vo
     a.xch = r.xch;
     a.epoch = r.epoch;
     a.err = ctx->err_dev;
+    a.wait_ns = r.wait_ns;
     ResConsts<T, NC> k = make_res_consts<T, NC>(ctx);
     ResSrc<T> sa{};
     if (src) {
@@ -899,7 +903,7 @@ dugks_status plan_flow(dugks_ctx* ctx) {
     if (ctx->precision != 32 || ctx->nc == NC_LARGE) return DUGKS_OK;
     const double slots = double(ctx->sms) * ctx->occupancy;
     const long long want = std::max<long long>(1, (long long)(DUGKS_FLOW_WAVES * slots / ctx->nstrips));
-    FlowPlan f{0, 0, ctx->nstrips, nullptr};
+    FlowPlan f{0, 0, ctx->nstrips, nullptr, kWaitNs};
     f.rows = int(std::max<long long>(std::min(DUGKS_FLOW_MIN_ROWS, ctx->ny), (ctx->ny + want - 1) / want));
     f.nseg = (ctx->ny + f.rows - 1) / f.rows;
     if ((long long)f.nstrips * f.nseg > INT_MAX / kFlowChunk) return DUGKS_OK;
@@ -912,9 +916,11 @@ dugks_status plan_flow(dugks_ctx* ctx) {
 }
 size_t flow_bytes(const FlowPlan& f) { return f.rows ? (1 + size_t(f.nstrips) * f.nseg) * sizeof(unsigned) : 0; }
 
+// skip: leave tile 0 of the first step out (dugks_tile_timeout_check)
 template <int NC>
-cudaError_t launch_flow(dugks_ctx* ctx, int n) {
+cudaError_t launch_flow(dugks_ctx* ctx, int n, bool skip = false) {
     cudaError_t e = cudaMemsetAsync(ctx->flow.sync, 0, flow_bytes(ctx->flow), ctx->stream);
+    if (e == cudaSuccess && skip) e = cudaMemsetAsync(ctx->flow.sync, 1, 1, ctx->stream);  // (one tile taken: low byte 1)
     if (e != cudaSuccess) return e;
     const unsigned grid = unsigned(n) * unsigned(ctx->flow.nstrips) * unsigned(ctx->flow.nseg);
     const int c = ctx->cur;
@@ -1908,6 +1914,30 @@ dugks_status dugks_wait_timeout_check(dugks_ctx* ctx, int limit_us) {
     wait_timeout_kernel<<<1, 32, 0, ctx->stream>>>(ctx->err_dev, 1000ull * (unsigned long long)limit_us);
     CK(cudaGetLastError());
     return DUGKS_OK;
+}
+
+dugks_status dugks_tile_timeout_check(dugks_ctx* ctx, int limit_us) {
+    if (!ctx || limit_us < 1 || limit_us > 1000000) return DUGKS_ERR_ARG;
+    DeviceGuard guard(ctx->device);
+    const unsigned long long ns = 1000ull * (unsigned long long)limit_us;
+    ResPlan& r = ctx->nsrc > 0 ? ctx->res_src : ctx->res;
+    if (r.ntx * r.nty > 1) {  // tile 0 counts its steps from elsewhere: nobody receives what it publishes
+        CK(cudaMemsetAsync(r.epoch, 0x40, sizeof(unsigned), ctx->stream));
+        r.wait_ns = ns;
+        const cudaError_t e = launch_resident_any(ctx, 2, ctx->buf[ctx->cur], ctx->buf[ctx->cur], nullptr);
+        r.wait_ns = kWaitNs;
+        CK(e);
+        return DUGKS_OK;
+    }
+    if (r.ntx == 0 && ctx->nsrc == 0 && ctx->flow.rows > 0) {
+        ctx->flow.wait_ns = ns;
+        const cudaError_t e = ctx->nc == 3 ? launch_flow<3>(ctx, 2, true) : launch_flow<4>(ctx, 2, true);
+        ctx->flow.wait_ns = kWaitNs;
+        CK(e);
+        return DUGKS_OK;
+    }
+    ctx->last_error = "no tiles of this context's step wait for one another";
+    return DUGKS_ERR_UNSUPPORTED;
 }
 
 dugks_status dugks_info(const dugks_ctx* ctx, dugks_info_t* out) {

@@ -94,6 +94,7 @@ struct ResArgs {
     uint4* xch;              // [2][tiles][res_slots][words]: published cells
     unsigned* epoch;         // [tiles]: steps done so far
     int* err;
+    unsigned long long wait_ns;  // limit of a wait for a neighbour's cell
 };
 
 constexpr int kResSrcChunk = 32;  // steps per launch with source terms (their time factors are launch arguments)
@@ -778,10 +779,10 @@ __global__ void __launch_bounds__(kResThreads<T>, 1)
                 unsigned long long t0 = 0, t1;
                 for (unsigned spin = 1;; ++spin) {
                     if (res_receive(p, P, phi, tag)) break;
-                    if ((spin & 255u) == 0) {  // give up after 2 s, or when another CTA has
+                    if ((spin & 255u) == 0) {  // give up after wait_ns, or when another CTA has
                         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
                         if (t0 == 0) t0 = t1;
-                        if (t1 - t0 > 2000000000ull || (*reinterpret_cast<volatile int*>(a.err) & 1)) {
+                        if (t1 - t0 > a.wait_ns || (*reinterpret_cast<volatile int*>(a.err) & 1)) {
                             fail = true;
                             break;
                         }

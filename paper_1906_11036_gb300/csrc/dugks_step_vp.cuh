@@ -439,6 +439,7 @@ __global__ void __launch_bounds__(32, DUGKS_SV_MIN_WARPS)
 struct FlowPlan {
     int rows, nseg, nstrips;
     unsigned* sync;  // [0]: tiles taken; [1 + tile]: steps done (all zero at launch)
+    unsigned long long wait_ns;  // limit of a wait for a neighbour
 };
 constexpr unsigned kFlowFailed = 0x80000000u;  // in sync[0] (a launch has fewer tiles): a wait expired
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
@@ -492,7 +493,7 @@ __global__ void __launch_bounds__(32, DUGKS_SV_MIN_WARPS)
                 if ((spin & 63u) == 0) {
                     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(w1));
                     if (w0 == 0) w0 = w1;
-                    if (w1 - w0 > 2000000000ull || (*reinterpret_cast<volatile int*>(a0.err) & 1)) {
+                    if (w1 - w0 > fp.wait_ns || (*reinterpret_cast<volatile int*>(a0.err) & 1)) {
                         ok = false;
                         break;
                     }

@@ -104,6 +104,7 @@ def library():
         L.dugks_set_stream.argtypes = [vp, vp]
         L.dugks_sync.argtypes = [vp]
         L.dugks_wait_timeout_check.argtypes = [vp, ctypes.c_int]
+        L.dugks_tile_timeout_check.argtypes = [vp, ctypes.c_int]
         L.dugks_set_adjoint_kernel.argtypes = [vp, ctypes.c_int]
         L.dugks_set_feq_check.argtypes = [vp, ctypes.c_int]
         L.dugks_info.argtypes = [vp, P(Info)]
@@ -148,7 +149,7 @@ def library():
         L.dugks_last_error.restype = ctypes.c_char_p
         for name in ("dugks_check_config", "dugks_create", "dugks_destroy", "dugks_init_phi", "dugks_init_phi_host",
                      "dugks_step", "dugks_get_phi", "dugks_get_phi_host", "dugks_save_state", "dugks_load_state",
-                     "dugks_set_stream", "dugks_sync", "dugks_wait_timeout_check", "dugks_info",
+                     "dugks_set_stream", "dugks_sync", "dugks_wait_timeout_check", "dugks_tile_timeout_check", "dugks_info",
                      "dugks_adjoint_step", "dugks_adjoint",
                      "dugks_set_source",
                      "dugks_phi_mass_noalloc", "dugks_batch_create", "dugks_batch_destroy", "dugks_batch_init_phi",
@@ -345,6 +346,10 @@ class Solver:
     def wait_timeout_check(self, limit_us: int = 2000):
         """Let one bounded device wait expire on purpose (no fault): the next sync raises DUGKS_ERR_TIMEOUT."""
         self._check(self.L.dugks_wait_timeout_check(self.h, int(limit_us)), "dugks_wait_timeout_check")
+
+    def tile_timeout_check(self, limit_us: int = 2000):
+        """Let the waits between the tiles of a many-step launch expire on purpose (no fault); then as above."""
+        self._check(self.L.dugks_tile_timeout_check(self.h, int(limit_us)), "dugks_tile_timeout_check")
 
     def set_feq_check(self, on: bool = True):
         """Later initialisations reject a negative equilibrium of phi0 (see dugks_check_feq)."""

@@ -59,3 +59,55 @@ def test_many_step_launches_after_an_expired_wait_leave_the_state(nx, ny, prec):
     assert ei.value.status == 7
     assert torch.equal(before, after)
     s.close()
+
+
+TILED = {"resident_fp32": lambda: (I.burgers(70, 45), 32), "resident_fp64": lambda: (I.burgers(64, 64), 64),
+         "resident_walls": lambda: (I.nonuniform(330, 517), 32), "resident_source": lambda: (I.cde_source(60), 32),
+         "sequence": lambda: (I.burgers(900, 700), 32), "sequence_walls": lambda: (I.nonuniform(1021, 643), 32)}
+
+
+@pytest.mark.parametrize("name", list(TILED))
+def test_a_tile_that_never_answers_ends_the_launch(name):
+    """One tile's messages (or its step count) never come: every tile's wait runs out, the launch ends by
+    itself, the status says so, and a fresh context computes what one that never failed does."""
+    import time
+
+    from paper_1906_11036_gb300.dugks import DugksError, Solver
+
+    (p, phi0), prec = TILED[name]()
+    phi0 = torch.tensor(phi0, device="cuda")
+    out = []
+    for fails in (True, False):
+        if fails:
+            s = Solver(p, precision=prec)
+            s.init_phi(phi0)
+            s.step(3)
+            s.sync()
+            t = time.perf_counter()
+            s.tile_timeout_check(2000)
+            with pytest.raises(DugksError) as ei:
+                s.sync()
+            assert ei.value.status == 7 and time.perf_counter() - t < 1.0
+            s.step(4)
+            with pytest.raises(DugksError) as ei:
+                s.get_phi_host()
+            assert ei.value.status == 7
+            s.close()
+        s = Solver(p, precision=prec)
+        s.init_phi(phi0)
+        s.step(7)
+        out.append(s.save_state())
+        s.sync()
+        s.close()
+    assert torch.equal(*out)
+
+
+def test_no_tiles_to_wait_for():
+    from paper_1906_11036_gb300.dugks import DugksError, Solver
+
+    p, _ = I.burgers(40, 30)
+    s = Solver(p, precision=32, kernel="naive")
+    with pytest.raises(DugksError) as ei:
+        s.tile_timeout_check(2000)
+    assert ei.value.status == 5
+    s.close()
