@@ -7,6 +7,7 @@ fallback.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 
@@ -440,8 +441,8 @@ class BatchSolver:
         if st != OK:
             raise DugksError(st, "dugks_batch_create")
         self.h, self.L, self.n = h, L, n
-        # the stream the batch runs on, and two events that order it with the caller's stream around
-        # an initialisation
+        # the stream the batch runs on, and two events that order it with the caller's stream around a call
+        # that takes or returns a tensor
         self._own = torch.cuda.ExternalStream(L.dugks_batch_stream(h), self.device)
         self._ready, self._taken = torch.cuda.Event(), torch.cuda.Event()
 
@@ -472,22 +473,34 @@ class BatchSolver:
         self._taken.record(self._own)
         caller.wait_event(self._taken)
 
+    @contextlib.contextmanager
+    def _result(self, *shape):
+        """A tensor that the batch's stream writes and the caller's reads.  Its memory belongs to the batch's
+        stream, so what the caller has queued cannot still be using it; the caller's stream waits for the write."""
+        caller = self.torch.cuda.current_stream(self.device)
+        with self.torch.cuda.stream(self._own):
+            out = self.torch.empty(shape, dtype=self.torch.float32, device=self.device)
+        yield out
+        out.record_stream(caller)
+        self._taken.record(self._own)
+        caller.wait_event(self._taken)
+
     def step(self, n: int = 1):
         self._check(self.L.dugks_batch_step(self.h, int(n)), "dugks_batch_step")
 
     def get_phi(self, i: int, mass: bool = False):
         p = self.problems[i]
-        out = self.torch.empty((p.ny, p.nx), dtype=self.torch.float32, device=self.device)
         m = ctypes.c_double(0.0)
-        self._check(self.L.dugks_batch_get_phi(self.h, int(i), ctypes.c_void_p(out.data_ptr()),
-                                               ctypes.byref(m) if mass else None), "dugks_batch_get_phi")
+        with self._result(p.ny, p.nx) as out:
+            self._check(self.L.dugks_batch_get_phi(self.h, int(i), ctypes.c_void_p(out.data_ptr()),
+                                                   ctypes.byref(m) if mass else None), "dugks_batch_get_phi")
         return (out, m.value) if mass else out
 
     def save_state(self, i: int):
         p = self.problems[i]
-        out = self.torch.empty((9, p.ny, p.nx), dtype=self.torch.float32, device=self.device)
-        self._check(self.L.dugks_batch_save_state(self.h, int(i), ctypes.c_void_p(out.data_ptr())),
-                    "dugks_batch_save_state")
+        with self._result(9, p.ny, p.nx) as out:
+            self._check(self.L.dugks_batch_save_state(self.h, int(i), ctypes.c_void_p(out.data_ptr())),
+                        "dugks_batch_save_state")
         return out
 
     def sync(self):
