@@ -53,8 +53,8 @@ enum { DUGKS_WALL_W = 0, DUGKS_WALL_E = 1, DUGKS_WALL_S = 2, DUGKS_WALL_N = 3 };
 enum { DUGKS_D2Q9 = 9 };
 enum { DUGKS_FP32 = 32, DUGKS_FP64 = 64 };
 enum {
-    DUGKS_KERNEL_AUTO = 0,  /* the fused streaming kernel */
-    DUGKS_KERNEL_FUSED = 1, /* fused streaming kernel: TMA row pipeline, one read and one write of ftilde */
+    DUGKS_KERNEL_AUTO = 0,  /* the fastest for the grid: many steps per launch where dugks_step says so, else as FUSED */
+    DUGKS_KERNEL_FUSED = 1, /* fused streaming kernel: TMA row pipeline, one read and one write of ftilde, a launch per step */
     DUGKS_KERNEL_NAIVE = 2  /* one thread per cell, everything recomputed from global memory (cross-check) */
 };
 
@@ -171,10 +171,12 @@ dugks_status dugks_init_phi(dugks_ctx *ctx, const void *phi0_dev);
 dugks_status dugks_init_phi_host(dugks_ctx *ctx, const double *phi0_host);
 
 /* Advance n >= 0 time steps (Eq. 2.12 with the interface flux of Eqs.
- * 2.19-2.22 and Eq. 2.9), asynchronously on the context's stream.  Grids whose
- * state fits in the SMs' shared memory (about 630^2 cells in FP32, 435^2 in
- * FP64) take up to 1024 steps per (cooperative) launch, or 32 with source
- * terms; larger FP32 grids up to 256; otherwise one launch per step. */
+ * 2.19-2.22 and Eq. 2.9), asynchronously on the context's stream.  With
+ * DUGKS_KERNEL_AUTO grids whose state fits in the SMs' shared memory (about
+ * 630^2 cells in FP32, 435^2 in FP64) take up to 1024 steps per (cooperative)
+ * launch, or 32 with source terms; larger FP32 grids up to 256 (calls of more
+ * than one step, no source terms, equilibria of degree <= 3); otherwise, and
+ * with the other kernels, one launch per step. */
 dugks_status dugks_step(dugks_ctx *ctx, long long n);
 
 /* phi = sum_i ftilde_i (text after Eq. 2.13) into phi_dev_out (device,

@@ -92,6 +92,7 @@ struct dugks_ctx {
     bool plain = false;                   // step_vp with the interior variant (long-segment plans)
     int nseg_sp_src = 0;
     SegPlan sp{1, 0, 1};  // step_vp: long segments first, then short ones
+    bool many = false;     // a launch may take many steps (resident step, flow_vp): DUGKS_KERNEL_AUTO
     ResPlan res, res_src;  // the resident step without and with source terms
     FlowPlan flow{0, 0, 0, nullptr, kWaitNs};  // flow_vp (rows = 0: not taken)
     bool flow_plain = false;          // with the interior variant
@@ -1588,6 +1589,7 @@ static dugks_status create_ctx(const dugks_mesh* mesh, const dugks_vset* vset, c
     ctx->ny = mesh->ny;
     ctx->precision = o.precision;
     ctx->kernel = o.kernel == DUGKS_KERNEL_NAIVE ? DUGKS_KERNEL_NAIVE : DUGKS_KERNEL_FUSED;
+    ctx->many = stepped_alone && o.kernel == DUGKS_KERNEL_AUTO;
     ctx->xper = mesh->bc[0] == DUGKS_BC_PERIODIC;
     ctx->yper = mesh->bc[2] == DUGKS_BC_PERIODIC;
     for (int w = 0; w < 4; ++w) ctx->bcv[w] = mesh->bc_value[w];
@@ -1640,8 +1642,8 @@ static dugks_status create_ctx(const dugks_mesh* mesh, const dugks_vset* vset, c
     };
     if (ctx->kernel == DUGKS_KERNEL_FUSED) {
         if ((st = plan_fused(ctx)) != DUGKS_OK) return fail(st);
-        if (stepped_alone && (st = plan_resident(ctx, 0, ctx->res)) != DUGKS_OK) return fail(st);
-        if (stepped_alone && ctx->res.ntx == 0 && (st = plan_flow(ctx)) != DUGKS_OK) return fail(st);
+        if (ctx->many && (st = plan_resident(ctx, 0, ctx->res)) != DUGKS_OK) return fail(st);
+        if (ctx->many && ctx->res.ntx == 0 && (st = plan_flow(ctx)) != DUGKS_OK) return fail(st);
     }
 
     const int lane = 128 / int(ctx->elem);  // rows padded to 128 bytes
@@ -2041,7 +2043,7 @@ dugks_status dugks_set_source(dugks_ctx* ctx, int nterms, const double* rate, co
                                fields + size_t(order[q]) * cells * ctx->elem, cells * ctx->elem,
                                cudaMemcpyDeviceToDevice, ctx->stream));
     }
-    if (nterms > 0) {  // (the stream is idle: see above)
+    if (nterms > 0 && ctx->many) {  // (the stream is idle: see above)
         dugks_status st = plan_resident(ctx, nterms, ctx->res_src);
         if (st != DUGKS_OK) return st;
         if (const size_t n = resident_bytes(ctx, ctx->res_src)) {
