@@ -706,7 +706,8 @@ def main():
     cells = p.nx * p.ny
     cvu_per_step = cells * Q * S
     stream = torch.cuda.Stream()
-    solver = Solver(p, precision=32, stream=stream)
+    # one step per call runs step_vp, a launch per step, like kernel "fused"; more run flow_vp
+    solver = Solver(p, precision=32, stream=stream, kernel="auto" if S > 1 else "fused")
     info = solver.info()
     with torch.cuda.stream(stream):
         solver.init_phi(torch.tensor(phi0, device="cuda"))
@@ -780,12 +781,12 @@ def main():
         "warmup": args.warmup, "ms_per_step": 1e3 * t_dev / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": config_dict(args, p),
-        "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": 8 * cells, "d2h_bytes_per_step": 8 * cells + 8},
-        "gpu_launches": args.steps * -(-S // FLOW_CHUNK),
+        "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": 8 * cells, "d2h_bytes_per_step": 8 * cells + 40},
+        "gpu_launches": args.steps * (-(-S // FLOW_CHUNK) if S > 1 else 1),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "traffic": profile_traffic(args.workload), "peak_kind": peak_kind,
                      "frac_of_nominal": achieved / NOMINAL_HBM_GBS, "nominal_peak": NOMINAL_HBM_GBS,
-                     "kernel": "flow_vp", "kernel_ms": step_s * 1e3,
+                     "kernel": "flow_vp" if S > 1 else "step_vp", "kernel_ms": step_s * 1e3,
                      "kernel_ms_from": "looped timing: interval time / time steps",
                      "kernel_ms_events": launch_s * 1e3,
                      "algorithmic_bytes_per_step": alg_bytes},

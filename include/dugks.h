@@ -118,7 +118,7 @@ typedef struct {
     long long steps_done;   /* time steps taken since the last init/load */
     double dt, lambda, cfl; /* time step, relaxation time alpha/c_s^2, c dt / min cell width */
     int block_threads;      /* threads per block of the step kernel */
-    int grid_blocks;        /* blocks per launch of the step kernel */
+    int grid_blocks;        /* blocks per launch of the step kernel (per step, where a launch takes tiles of many) */
     long long state_bytes;  /* bytes of one ftilde buffer (two are held) */
     double time;            /* time of the current state (source terms only; see dugks_set_source) */
     int nsrc;               /* source terms set */

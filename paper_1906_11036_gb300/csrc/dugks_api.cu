@@ -934,6 +934,12 @@ cudaError_t launch_flow(dugks_ctx* ctx, int n, bool skip = false) {
     return cudaGetLastError();
 }
 
+// row segments (per strip) of the row-marching kernel that dugks_step runs
+int row_segments(const dugks_ctx* ctx) {
+    if (ctx->nsrc > 0) return ctx->precision == 32 && ctx->nc != NC_LARGE ? ctx->nseg_sp_src : ctx->nseg_src;
+    return ctx->flow.rows > 0 ? ctx->flow.nseg : ctx->nseg;
+}
+
 // steps a resident launch may take (0: the grid runs the row-marching kernels)
 long long resident_chunk(const dugks_ctx* ctx) {
     if ((ctx->nsrc > 0 ? ctx->res_src : ctx->res).ntx == 0) return 0;
@@ -1956,7 +1962,7 @@ dugks_status dugks_info(const dugks_ctx* ctx, dugks_info_t* out) {
     const ResPlan& r = ctx->nsrc > 0 ? ctx->res_src : ctx->res;
     out->block_threads = ctx->kernel == DUGKS_KERNEL_NAIVE ? 128 : (r.ntx > 0 ? r.threads : ctx->nt);
     out->grid_blocks = ctx->kernel == DUGKS_KERNEL_NAIVE ? ((ctx->nx + 127) / 128) * std::min(ctx->ny, 65535)
-                                                         : (r.ntx > 0 ? r.ntx * r.nty : ctx->nstrips * ctx->nseg);
+                                                         : (r.ntx > 0 ? r.ntx * r.nty : ctx->nstrips * row_segments(ctx));
     out->state_bytes = (long long)Q * ctx->plane * (long long)ctx->elem;
     out->time = ctx->t;
     out->nsrc = ctx->nsrc;

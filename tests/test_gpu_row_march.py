@@ -95,3 +95,14 @@ def test_gradient(walls, prec, every):
     else:
         assert float((g1 - g2).norm() / g2.norm()) <= 1e-11 and abs(a1 - a2) <= 1e-11 * abs(a2)
         assert np.abs(np.subtract(u1, u2)).max() <= 1e-11 * np.abs(u2).max()
+
+
+def test_info_gives_the_grid_that_runs():
+    """grid_blocks: 30-column strips times the row segments of the kernel that steps (the tile sequence's with
+    AUTO on a large FP32 grid, the row march's own with "fused")."""
+    p, _ = I.burgers(900, 700)
+    a, f = (_solver(p, 32, k) for k in ("auto", "fused"))
+    na, nf = a.info()["grid_blocks"], f.info()["grid_blocks"]
+    a.close()
+    f.close()
+    assert na % 30 == 0 and nf % 30 == 0 and na > nf
