@@ -2107,26 +2107,33 @@ dugks_status dugks_adjoint(dugks_ctx* ctx, const void* phi0_dev, long long nstep
     const long long K = std::min<long long>(checkpoint_every, std::max<long long>(nsteps, 1));
     const long long nseg = nsteps == 0 ? 0 : (nsteps + K - 1) / K;
     // one workspace: the states at the segment starts after the first (the first is the context's own
-    // state buffer) and the states of a segment after its start, laid out like the context's
-    // buffers, and two lambdas
-    const size_t sbytes = size_t(Q) * ctx->plane * ctx->elem;
+    // state buffer) and the states of a segment after its start, and two lambdas.  The states are laid
+    // out like the context's buffers, so that steps read and write them in place, or (packed), where the
+    // device has no room for the padded rows, contiguously, with a copy to and from the context's buffers
     const size_t lbytes = (size_t(Q) * ctx->nx * ctx->ny * ctx->elem + 255) / 256 * 256;
     const long long nck = std::max<long long>(nseg - 1, 0), nst = nck + K - 1;
-    const size_t at_lam = (sbytes * size_t(nst) + 255) / 256 * 256;
-    const size_t need = at_lam + 2 * lbytes;
-    if (need > ctx->adj_ws_bytes) {
+    bool packed = false;
+    size_t sbytes = size_t(Q) * ctx->plane * ctx->elem, at_lam = 0;
+    for (;; packed = true, sbytes = lbytes) {
+        at_lam = (sbytes * size_t(nst) + 255) / 256 * 256;
+        const size_t need = at_lam + 2 * lbytes;
+        if (need <= ctx->adj_ws_bytes) break;
         if (ctx->adj_ws) {
             cudaStreamSynchronize(ctx->stream);
             cudaFree(ctx->adj_ws);
             ctx->adj_ws = nullptr;
             ctx->adj_ws_bytes = 0;
         }
-        if (cudaMalloc(&ctx->adj_ws, need) != cudaSuccess) {
-            ctx->adj_ws = nullptr;
+        if (cudaMalloc(&ctx->adj_ws, need) == cudaSuccess) {
+            ctx->adj_ws_bytes = need;
+            break;
+        }
+        ctx->adj_ws = nullptr;
+        cudaGetLastError();
+        if (packed) {
             ctx->last_error = "adjoint workspace allocation failed";
             return DUGKS_ERR_NOMEM;
         }
-        ctx->adj_ws_bytes = need;
     }
     unsigned char* ws = static_cast<unsigned char*>(ctx->adj_ws);
     std::vector<void*> state(size_t(nst) + 1, nullptr);  // [0]: step 0, [1 .. nck]: segment starts, then the segment
@@ -2142,14 +2149,25 @@ dugks_status dugks_adjoint(dugks_ctx* ctx, const void* phi0_dev, long long nstep
     if ((st = dugks_init_phi(ctx, phi0_dev)) != DUGKS_OK) return st;
     state[0] = ctx->buf[ctx->cur];
     std::vector<CUtensorMap> map(state.size());
-    if (ctx->kernel == DUGKS_KERNEL_FUSED && (st = make_state_maps(ctx, state.data(), int(state.size()), map.data())) != DUGKS_OK)
+    if (!packed && ctx->kernel == DUGKS_KERNEL_FUSED &&
+        (st = make_state_maps(ctx, state.data(), int(state.size()), map.data())) != DUGKS_OK)
         return st;
     auto step = [&](long long from, long long to) {  // one row-marching step between two states
         return launch_step_any(ctx, StepIO{state[size_t(from)], state[size_t(to)], &map[size_t(from)]});
     };
+    // packed: the context's buffers to state `from`
+    auto load = [&](long long from) { return from == 0 ? dugks_init_phi(ctx, phi0_dev) : dugks_load_state(ctx, state[size_t(from)]); };
     // n steps from state `from` to state `to`, the states in between (keep) in seg[1 .. n - 1], or
     // there only for a while; a resident launch keeps them as it goes
     auto advance = [&](long long from, long long to, long long n, bool keep) -> cudaError_t {
+        if (packed) {
+            dugks_status s = load(from);
+            for (long long m = 1; m <= n && s == DUGKS_OK; ++m) {
+                s = dugks_step(ctx, 1);
+                if (s == DUGKS_OK && (keep || m == n)) s = dugks_save_state(ctx, m == n ? state[size_t(to)] : seg[m]);
+            }
+            return s == DUGKS_OK ? cudaSuccess : cudaErrorUnknown;
+        }
         const long long chunk = resident_chunk(ctx);
         if (chunk > 0) {
             cudaError_t r = cudaSuccess;
@@ -2196,7 +2214,12 @@ dugks_status dugks_adjoint(dugks_ctx* ctx, const void* phi0_dev, long long nstep
         if (ns > 1 && (e = advance(s, nck + ns - 1, ns - 1, true)) != cudaSuccess) return fail(e, "recomputed segment");
         for (long long q = ns - 1; q >= 0; --q) {
             const void* f = q == 0 ? state[size_t(s)] : seg[q];
-            if ((e = launch_adjoint_step_any(ctx, f, ctx->pitch, lam[cur], lam[1 - cur], nullptr, nullptr, want_u, true,
+            if (packed && s == 0 && q == 0) {  // step 0 again: the context's buffers have moved on from it
+                if ((st = load(0)) != DUGKS_OK) return st;
+                f = ctx->buf[ctx->cur];
+            }
+            const long long pitch = packed && (s > 0 || q > 0) ? ctx->nx : ctx->pitch;
+            if ((e = launch_adjoint_step_any(ctx, f, pitch, lam[cur], lam[1 - cur], nullptr, nullptr, want_u, true,
                                              true)) != cudaSuccess)
                 return fail(e, "adjoint step");
             cur ^= 1;
