@@ -68,6 +68,7 @@ dugks_status fail3(dugks_3d_ctx* ctx, cudaError_t e, const char* what) {
         snprintf(b, sizeof(b), "%s: %s", what, cudaGetErrorString(e));
         ctx->last_error = b;
     }
+    cudaGetLastError();  // reported here: the next launch's check is not to find it again
     return e == cudaErrorMemoryAllocation ? DUGKS_ERR_NOMEM : DUGKS_ERR_CUDA;
 }
 

@@ -157,6 +157,7 @@ dugks_status cuda_fail(dugks_ctx* ctx, cudaError_t e, const char* what) {
     if (ctx) {
         ctx->last_error = std::string(what) + ": " + cudaGetErrorString(e);
     }
+    cudaGetLastError();  // reported here: the next launch's check is not to find it again
     return e == cudaErrorMemoryAllocation ? DUGKS_ERR_NOMEM : DUGKS_ERR_CUDA;
 }
 
@@ -1370,6 +1371,7 @@ dugks_status batch_fail(dugks_batch* b, cudaError_t e, const char* what) {
     char buf[256];
     snprintf(buf, sizeof(buf), "%s: %s", what, cudaGetErrorString(e));
     b->last_error = buf;
+    cudaGetLastError();
     return e == cudaErrorMemoryAllocation ? DUGKS_ERR_NOMEM : DUGKS_ERR_CUDA;
 }
 
