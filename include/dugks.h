@@ -242,7 +242,9 @@ dugks_status dugks_info(const dugks_ctx *ctx, dugks_info_t *out);
  * source).  t0 is the time of the current state and of every later
  * dugks_init_phi; each step advances it by dt (dugks_info_t.time).
  * Errors: DUGKS_ERR_ARG (bad counts, null pointers, non-finite rates or t0),
- * DUGKS_ERR_UNSUPPORTED (C = 0, or the naive kernel), DUGKS_ERR_NOMEM.
+ * DUGKS_ERR_UNSUPPORTED (C = 0, or the naive kernel), both before anything
+ * changes; DUGKS_ERR_NOMEM or DUGKS_ERR_CUDA, which leave the context without
+ * a source.
  * The adjoint and batched entry points refuse a context with a source. */
 dugks_status dugks_set_source(dugks_ctx *ctx, int nterms, const double *rate, const int *power,
                               const void *fields_dev, double t0);

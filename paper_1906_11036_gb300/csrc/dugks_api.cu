@@ -584,10 +584,10 @@ void set_resident_buffers(const dugks_ctx* ctx, ResPlan& r, void* p) {
 // FP64 64^2 150 / 4.7, 200^2 172 / 23, 400^2 155 / 59, 430^2 163 / 70.
 dugks_status plan_resident(dugks_ctx* ctx, int nsrc, ResPlan& r) {
     free_resident(r);
-    int sms = 0, smem_max = 0, coop = 0;
+    const int sms = ctx->sms;
+    int smem_max = 0, coop = 0;
     cudaError_t e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device)) != cudaSuccess ||
-        (e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device)) != cudaSuccess ||
+    if ((e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device)) != cudaSuccess)
         return cuda_fail(ctx, e, "cudaDeviceGetAttribute");
     if (!coop) return DUGKS_OK;
@@ -1992,8 +1992,11 @@ dugks_status dugks_set_source(dugks_ctx* ctx, int nterms, const double* rate, co
     for (int q = 0; q < nterms; ++q) order[q] = q;
     std::stable_sort(order, order + nterms, [&](int x, int y) { return power[x] < power[y]; });
     const char* fields = static_cast<const char*>(fields_dev);
-    if (nterms > 0 && src_uses_aux(ctx)) {
+    if (nterms > 0) {
         CK(cudaStreamSynchronize(ctx->stream));  // the old fields may still be read by queued steps
+        ctx->nsrc = 0;                           // their buffers go first: a call that fails below leaves no source
+    }
+    if (nterms > 0 && src_uses_aux(ctx)) {
         EncodeTiledFn encode = tiled_encoder(ctx);
         if (!encode) return DUGKS_ERR_CUDA;
         using L = WarpLayout<float>;
@@ -2037,7 +2040,6 @@ dugks_status dugks_set_source(dugks_ctx* ctx, int nterms, const double* rate, co
                 plan_long_short(ctx, (long long)sms * occ, kSrcPlanFirst, kSrcPlanShort, ctx->sp_src, ctx->nseg_sp_src);
         }
     } else if (nterms > 0) {
-        CK(cudaStreamSynchronize(ctx->stream));  // the old fields may still be read by queued steps
         if (ctx->src_field) { cudaFree(ctx->src_field); ctx->src_field = nullptr; }
         cudaError_t e = cudaMalloc(&ctx->src_field, size_t(nterms) * cells * ctx->elem);
         if (e != cudaSuccess) { ctx->src_field = nullptr; return cuda_fail(ctx, e, "cudaMalloc(source fields)"); }
