@@ -175,7 +175,7 @@ dugks_status dugks_init_phi_host(dugks_ctx *ctx, const double *phi0_host);
  * DUGKS_KERNEL_AUTO grids whose state fits in the SMs' shared memory (about
  * 630^2 cells in FP32, 435^2 in FP64) take up to 1024 steps per (cooperative)
  * launch, or 32 with source terms; larger FP32 grids up to 256 (calls of more
- * than one step, no source terms, equilibria of degree <= 3); otherwise, and
+ * than a few steps, no source terms, equilibria of degree <= 3); otherwise, and
  * with the other kernels, one launch per step. */
 dugks_status dugks_step(dugks_ctx *ctx, long long n);
 

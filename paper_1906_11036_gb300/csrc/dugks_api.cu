@@ -96,6 +96,7 @@ struct dugks_ctx {
     ResPlan res, res_src;  // the resident step without and with source terms
     FlowPlan flow{0, 0, 0, nullptr, kWaitNs};  // flow_vp (rows = 0: not taken)
     bool flow_plain = false;          // with the interior variant
+    int flow_least = 2;               // steps a call takes for it at least
     long long steps_done = 0;
     // adjoint work buffers (allocated on first use)
     void* adj_ax = nullptr;
@@ -899,7 +900,23 @@ void* flow_fn(bool plain) {
     return plain ? reinterpret_cast<void*>(&flow_vp<NC, true>) : reinterpret_cast<void*>(&flow_vp<NC, false>);
 }
 
-// Every FP32 grid that does not take the resident step takes flow_vp for calls of more than one step
+// Steps from which a launch of flow_vp is the faster one.  Its first and last tiles leave the GPU partly
+// idle for about half a step, once per launch, against what each step_vp launch loses to its own: most
+// where its segments fill well under a wave of warps or a little over one, little where they nearly fill
+// one, least with long segments and interior warps (walls, where few warps then take the general routine).
+// Time of a call relative to single launches, over 36 grids of 0.4 to 9 M cells:
+//   waves < 0.6: 2 steps 0.85 ... 1.06 (once 1.14), 3 steps 0.77 ... 1.02
+//   0.6 ... 1:   2 steps 1.05 ... 1.20, 3 steps 0.94 ... 1.09, 4 steps 0.90 ... 1.04
+//   above 1:     2 steps 0.95 ... 1.06, 3 steps 0.87 ... 0.98
+//   long segments, periodic: 3 steps 0.96 ... 1.06, 5 steps 0.90 ... 1.02
+//   long segments, walls:    5 steps 0.90 ... 1.05, 8 steps 0.87 ... 1.03, 16 steps 0.85 ... 1.01
+int flow_least_steps(const dugks_ctx* ctx) {
+    if (ctx->plain) return ctx->xper && ctx->yper ? 5 : 12;
+    const double waves = double(ctx->nstrips) * ctx->nseg / (double(ctx->sms) * ctx->occupancy);
+    return waves < 0.6 ? 2 : waves <= 1.0 ? 4 : 3;
+}
+
+// Every FP32 grid that does not take the resident step takes flow_vp for calls of flow_least steps and more
 // (equilibria of degree <= 3, no source terms); tiles are counted in 32 bits.
 dugks_status plan_flow(dugks_ctx* ctx) {
     if (ctx->precision != 32 || ctx->nc == NC_LARGE) return DUGKS_OK;
@@ -910,6 +927,7 @@ dugks_status plan_flow(dugks_ctx* ctx) {
     f.nseg = (ctx->ny + f.rows - 1) / f.rows;
     if ((long long)f.nstrips * f.nseg > INT_MAX / kFlowChunk) return DUGKS_OK;
     ctx->flow_plain = f.rows >= DUGKS_FLOW_PLAIN_ROWS;
+    ctx->flow_least = flow_least_steps(ctx);
     void* fn = ctx->nc == 3 ? flow_fn<3>(ctx->flow_plain) : flow_fn<4>(ctx->flow_plain);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(fused_smem(ctx)));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute");
@@ -1812,7 +1830,7 @@ dugks_status dugks_step(dugks_ctx* ctx, long long n) {
                 continue;
             }
             CK(e);
-        } else if (ctx->flow.rows > 0 && ctx->nsrc == 0 && n - s > 1) {
+        } else if (ctx->flow.rows > 0 && ctx->nsrc == 0 && n - s >= ctx->flow_least) {
             m = std::min<long long>(n - s, kFlowChunk);
             CK(ctx->nc == 3 ? launch_flow<3>(ctx, int(m)) : launch_flow<4>(ctx, int(m)));
             ctx->cur ^= int(m & 1);
