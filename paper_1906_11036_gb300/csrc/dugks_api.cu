@@ -539,7 +539,10 @@ dugks_status plan_fused(dugks_ctx* ctx) {
 }
 
 // cost of a cell, of a face and of the start of a march: warp instructions in FP32, in FP64 the
-// instructions of its slow pipe
+// instructions of its slow pipe.  The tilings that plan_resident picks by them against the fastest of all
+// it could pick, each timed (us per step): FP32 70x45 1.84 / 1.75, 128^2 2.28 / 2.23, 200^2 2.84 / 2.84,
+// 330x517 4.85 / 4.80, 400^2 4.64 / 4.60, 512^2 6.26 / 6.25, 600^2 8.04 / 8.03, 1500x200 7.46 / 7.01; FP64
+// 64^2 5.44 / 5.36, 200^2 23.8 / 22.8, 400^2 72.6 / 71.6 (the median tiling takes 1.1 to 2.7 times as long)
 constexpr double kResCost[2][3] = {{120.0, 80.0, 45.0}, {75.0, 75.0, 2.0}};
 constexpr int kResChunk = 1024;  // steps per launch of the resident kernel at most
 
@@ -577,12 +580,14 @@ void set_resident_buffers(const dugks_ctx* ctx, ResPlan& r, void* p) {
 // Tiles of the resident step for nsrc source terms, at most one per SM, and the length of its
 // marches over faces, with the least time per step on one SM: the passes of its warps over cells
 // and over groups of 31 marches, weighed by the instructions of a cell, of a face and of the start
-// of a march.  A grid whose tiles do not fit in shared memory (above about 630^2 cells in FP32 and
-// 435^2 in FP64), or whose tiles are so thin that a CTA has too few threads for their outer
-// neighbours, keeps the row-marching kernels.  Up to that line the resident step was the faster one
-// wherever both were measured (us per step, row-marching against resident): FP32 70x45 20.5 / 1.8,
-// 200^2 with a source term 34 / 3.1, 330x517 16.6 / 4.7, 512^2 18.8 / 6.1, 620^2 20.9 / 8.6;
-// FP64 64^2 150 / 4.7, 200^2 172 / 23, 400^2 155 / 59, 430^2 163 / 70.
+// of a march.  Tilings whose largest tile has over 5/4 of the fewest cells possible are left out (the
+// fastest one never was among them), and so are tiles of over 8192 cells, which no shared memory holds.
+// A grid whose tiles do not fit in shared memory (above about 630^2 cells in FP32 and 435^2 in FP64), or
+// whose tiles are so thin that a CTA has too few threads for their outer neighbours, keeps the
+// row-marching kernels.  Up to that line the resident step was the faster one wherever both were measured
+// (us per step of a call of 50, row-marching against resident): FP32 70x45 20.5 / 2.1, 200^2 with a source
+// term 34.8 / 3.0, 330x517 16.4 / 5.0, 512^2 18.5 / 6.4, 620^2 20.5 / 9.1; FP64 64^2 160 / 5.6, 200^2
+// 172 / 22.5, 400^2 164 / 73.  A call of one step is faster too, or as fast within 2 us (620^2 22.5 to 20.5).
 dugks_status plan_resident(dugks_ctx* ctx, int nsrc, ResPlan& r) {
     free_resident(r);
     const int sms = ctx->sms;
@@ -880,19 +885,12 @@ cudaError_t launch_resident_any(dugks_ctx* ctx, int n, const void* in, void* out
 // Tiles of flow_vp per resident warp, and rows per tile at least.  More tiles than warps hide the start
 // and the end of a tile behind others, but each passes two rows more than it owns (us per step for
 // 1.4, 1.7, 2.0, 2.8 tiles per warp: 2048^2 tanh mesh 59.9, 60.8, 61.7, 67.3; 2048^2 periodic 74.0,
-// 64.8, 64.2, 69.3; 1024^2 23.1, 21.2, 21.7, 21.8).  On grids too small for that, short tiles keep the
-// chain of a step short (800x700: 10 rows 21.7, 8 20.2, 6 17.7, 4 16.4).
+// 64.8, 64.2, 69.3; 1024^2 23.1, 21.2, 21.7, 21.8; at 1.75, taken, 60.9, 64.0 and 21.1).  On grids too small
+// for that, short tiles keep the chain of a step short (800x700: 10 rows 21.7, 8 20.2, 6 17.7, 4 16.4).
 // One launch per step (step_vp) took 64.4, 76.1, 25.8 and 20.6 us on these grids.
-#ifndef DUGKS_FLOW_WAVES
-#define DUGKS_FLOW_WAVES 1.75
-#endif
-#ifndef DUGKS_FLOW_MIN_ROWS
-#define DUGKS_FLOW_MIN_ROWS 4
-#endif
-// rows per tile from which the interior variant of the row routine pays (see step_vp)
-#ifndef DUGKS_FLOW_PLAIN_ROWS
-#define DUGKS_FLOW_PLAIN_ROWS 24
-#endif
+constexpr double kFlowWaves = 1.75;
+constexpr int kFlowMinRows = 4;
+constexpr int kFlowPlainRows = 24;  // rows per tile from which the interior variant of the row routine pays (see step_vp)
 constexpr int kFlowChunk = 256;  // steps per launch at most
 
 template <int NC>
@@ -921,12 +919,12 @@ int flow_least_steps(const dugks_ctx* ctx) {
 dugks_status plan_flow(dugks_ctx* ctx) {
     if (ctx->precision != 32 || ctx->nc == NC_LARGE) return DUGKS_OK;
     const double slots = double(ctx->sms) * ctx->occupancy;
-    const long long want = std::max<long long>(1, (long long)(DUGKS_FLOW_WAVES * slots / ctx->nstrips));
+    const long long want = std::max<long long>(1, (long long)(kFlowWaves * slots / ctx->nstrips));
     FlowPlan f{0, 0, ctx->nstrips, nullptr, kWaitNs};
-    f.rows = int(std::max<long long>(std::min(DUGKS_FLOW_MIN_ROWS, ctx->ny), (ctx->ny + want - 1) / want));
+    f.rows = int(std::max<long long>(std::min(kFlowMinRows, ctx->ny), (ctx->ny + want - 1) / want));
     f.nseg = (ctx->ny + f.rows - 1) / f.rows;
     if ((long long)f.nstrips * f.nseg > INT_MAX / kFlowChunk) return DUGKS_OK;
-    ctx->flow_plain = f.rows >= DUGKS_FLOW_PLAIN_ROWS;
+    ctx->flow_plain = f.rows >= kFlowPlainRows;
     ctx->flow_least = flow_least_steps(ctx);
     void* fn = ctx->nc == 3 ? flow_fn<3>(ctx->flow_plain) : flow_fn<4>(ctx->flow_plain);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(fused_smem(ctx)));

@@ -239,11 +239,9 @@ __device__ __forceinline__ void res_moments(const PT (&P)[4], T& mx, T& my) {
 // weights of a face in shared memory: normal weights of the left and of the right cell for a pair
 // that moves along the normal (4), 1 - w, w, hcd, hc tl, hc tr; in FP64 the first four and a second
 // pair of tangential weights carry the factor a_f of Eq. 2.22 (one multiplication less per value)
-// faces of a march unrolled: 2 (512^2 FP32 6.11 us per step, 70x45 1.84) against 1 (6.35, 1.74)
-#ifndef DUGKS_RES_UNROLL
-#define DUGKS_RES_UNROLL 2
-#endif
-constexpr int kResUnroll = DUGKS_RES_UNROLL;
+// faces of a march unrolled: 2 (us per step: 512^2 FP32 6.25, 330x517 with walls 4.84, 400^2 4.64) against
+// 1 (6.35, 4.88, 4.56)
+constexpr int kResUnroll = 2;
 template <typename T>
 constexpr int kResFace = sizeof(T) == 4 ? 9 : 11;
 
@@ -401,16 +399,11 @@ __device__ __forceinline__ void res_cell_parts(const ResArgs<T>& a, const ResCon
     }
 }
 
-// threads per CTA at most.  FP32: 512 at 128 registers (512^2 6.3 us per step; 640 at 96 registers 6.7, 768 at
-// 80 8.1, 384 6.8).  FP64: 256, eight warps keep its pipe busy.
-#ifndef DUGKS_RES_THREADS32
-#define DUGKS_RES_THREADS32 512
-#endif
-#ifndef DUGKS_RES_THREADS64
-#define DUGKS_RES_THREADS64 256
-#endif
+// threads per CTA at most.  FP32: 512 at 128 registers (us per step at 70x45, 400^2, 512^2: 1.83, 4.64, 6.25;
+// 384 1.72, 4.44, 7.08; 640 at 96 registers 1.97, 5.43, 8.86; 768 at 80 2.34, 6.54, 11.4).  FP64: 256, eight
+// warps keep its pipe busy.
 template <typename T>
-constexpr int kResThreads = sizeof(T) == 4 ? DUGKS_RES_THREADS32 : DUGKS_RES_THREADS64;
+constexpr int kResThreads = sizeof(T) == 4 ? 512 : 256;
 
 template <typename T, int NC, bool SRC>
 __global__ void __launch_bounds__(kResThreads<T>, 1)
