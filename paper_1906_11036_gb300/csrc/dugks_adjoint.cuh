@@ -556,16 +556,18 @@ __global__ void __launch_bounds__(TX * TY) adj_tile_kernel(const StepArgs<T, NC>
         dfeq_all(ka, phi, dfe);
         // the moving velocities over the rest velocity (mu already is): the weights of Pb[0] and of mu[0]
         // sum to one over Eqs. 2.21 and 2.13 and the equilibria, so lam_0 takes them whole
-        T l0 = Pb[0] + mu[0], s = T(0), w[Q];
+        T pb = T(0), s = T(0), w[Q];  // (pb is small beside lam_0: summed first, it costs one rounding of it)
+        const T z = Pb[0] + mu[0];
 #pragma unroll
         for (int i = 1; i < Q; ++i) {
             Pb[i] -= Pb[0];
             w[i] = fma(ka.b_bp, Pb[i], ka.b_tp * mu[i]);
-            l0 = fma(w[i], dfe[i], l0);
+            pb = fma(w[i], dfe[i], pb);
             s += Pb[i] * fma(ka.da_bp, ft[i], ka.db_bp * fe[i]) + mu[i] * fma(ka.da_tp, ft[i], ka.db_tp * fe[i]);
         }
         djdl += double(s);
         if (g.want_u) add_du(ka, phi, w, kAllQ, du);  // Eqs. 2.21 and 2.13: b_bp feq(phi) in P and b_tp feq(phi) in ftilde^+
+        const T l0 = z + pb;
         g.lam[t] = l0;
 #pragma unroll
         for (int i = 1; i < Q; ++i) g.lam[i * cplane + t] = fma(ka.a_bp, Pb[i], ka.a_tp * mu[i]) + (g.dev ? T(0) : l0);

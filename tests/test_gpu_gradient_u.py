@@ -51,3 +51,29 @@ def test_dj_du_of_the_gradient(name, kind, seed):
     err = np.abs(np.subtract(u3, u6)).max() / np.abs(u6).max()
     assert float((g3.double() - g6).norm() / g6.norm()) <= 2e-6
     assert err <= 1e-6
+
+
+@pytest.mark.parametrize("name", ["periodic_512", "walls_2048x128"])
+def test_tiled_dj_dphi0_is_as_exact_as_the_row_kernels(name):
+    """Both FP32 kernels round lambda_0 the same few times a step, so their distances from 64 bits are the same
+    but for the order of their sums: within a quarter."""
+    import __graft_entry__
+
+    __graft_entry__.build()
+    from paper_1906_11036_gb300.dugks import Solver
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    p = CASES[name]()
+    xc, yc = p.centres()
+    phi0 = torch.tensor(I.smooth_phi0(xc, yc, seed=1), device="cuda").float()
+    misfit = torch.tensor(I.smooth_phi0(xc, yc, seed=21) - 0.9, device="cuda").float()
+    g = {}
+    for prec, kind in ((64, "tiled"), (32, "tiled"), (32, "rows")):
+        s = Solver(p, precision=prec)
+        s.set_adjoint_kernel(kind)
+        g[prec, kind] = s.gradient(phi0.to(s.dtype), 20, misfit.to(s.dtype), checkpoint_every=20)[0].double()
+        s.close()
+    ref = g[64, "tiled"]
+    tiled, rows = (float((g[32, k] - ref).norm() / ref.norm()) for k in ("tiled", "rows"))
+    assert tiled <= 1.25 * rows, (tiled, rows)
