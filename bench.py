@@ -55,7 +55,7 @@ KERNEL_SOURCES = [os.path.join(ROOT, "paper_1906_11036_gb300", "csrc", f)
                   for f in ("dugks_step_vp.cuh", "dugks_kernels.cuh", "dugks_device.cuh")]
 NOMINAL_HBM_GBS = 7900.0  # GB300 HBM3e, nominal
 FLOW_CHUNK = 256  # time steps per launch of flow_vp at most (kFlowChunk)
-FLOW_LEAST = {"nonuniform": 12, "burgers": 5}  # and of a call that takes it (flow_least_steps)
+FLOW_LEAST = {"nonuniform": 12, "burgers": 4}  # and of a call that takes it (flow_least_steps)
 
 
 def workload(name: str):
@@ -787,7 +787,7 @@ def main():
         "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": 8 * cells, "d2h_bytes_per_step": 8 * cells + 40},
         "gpu_launches": args.steps * (S // FLOW_CHUNK + (1 if S % FLOW_CHUNK >= flow_least else S % FLOW_CHUNK)),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                     "traffic": profile_traffic(args.workload), "peak_kind": peak_kind,
+                     "traffic": profile_traffic(args.workload) if flow else None, "peak_kind": peak_kind,
                      "frac_of_nominal": achieved / NOMINAL_HBM_GBS, "nominal_peak": NOMINAL_HBM_GBS,
                      "kernel": "flow_vp" if flow else "step_vp", "kernel_ms": step_s * 1e3,
                      "kernel_ms_from": "looped timing: interval time / time steps",

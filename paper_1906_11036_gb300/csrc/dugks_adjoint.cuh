@@ -567,10 +567,16 @@ __global__ void __launch_bounds__(TX * TY) adj_tile_kernel(const StepArgs<T, NC>
         }
         djdl += double(s);
         if (g.want_u) add_du(ka, phi, w, kAllQ, du);  // Eqs. 2.21 and 2.13: b_bp feq(phi) in P and b_tp feq(phi) in ftilde^+
-        const T l0 = z + pb;
-        g.lam[t] = l0;
+        g.lam[t] = z + pb;
+        if (g.dev) {
 #pragma unroll
-        for (int i = 1; i < Q; ++i) g.lam[i * cplane + t] = fma(ka.a_bp, Pb[i], ka.a_tp * mu[i]) + (g.dev ? T(0) : l0);
+            for (int i = 1; i < Q; ++i) g.lam[i * cplane + t] = fma(ka.a_bp, Pb[i], ka.a_tp * mu[i]);
+        } else {  // lam_0 + the deviation, with a_tp of plain mu as the one large term
+            const T base = fma(ka.b_tp, mu[0], Pb[0]) + pb;
+#pragma unroll
+            for (int i = 1; i < Q; ++i)
+                g.lam[i * cplane + t] = fma(ka.a_tp, g.mu[i * cplane + t], fma(ka.a_bp, Pb[i], base));
+        }
     }
     const double v[3] = {djdl, du[0], du[1]};
     block_partial3(v, g.partial + blockIdx.y * gridDim.x + blockIdx.x, g.pstride, g.accumulate);
